@@ -347,56 +347,77 @@ constexpr int lines_static() {
     return m;
 }
 
+// x pass, forward, two real rows per complex line: with z = a + i b for rows a, b
+// and Z its transform, A_k = (Z_k + conj Z_{N-k})/2 and B_k = (Z_k - conj Z_{N-k})/2i.
+// One transform serves two rows, so a pass costs half the butterflies of one
+// that sets the imaginary part to zero (FP64 is bound by them on GB300: the whole
+// 192 x 192 x 384 FP64 solve took 3.15 ms with one row per line, 2.56 ms with two;
+// 128 x 128 x 256 in FP32 0.137 and 0.125 ms). The rows of a pair are neighbours
+// (ny is even for every extent the library takes).
+// The first nkeep coefficients of each row go to C, rows `pitch` apart.
 template <typename T, int N, int M>
-__global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src, Cx<T>* C) {
+__global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src, Cx<T>* C, int nkeep, int pitch) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
-    constexpr int nxh = N / 2 + 1;
     Cx<T>* A = sw + N;
     Cx<T>* B = A + N * (M + 1);
     load_tw(sw, tw, N);
-    const long rows = (long)g.ny * g.nz;
-    const long row0 = (long)blockIdx.x * M;
+    const long pairs = (long)g.ny * g.nz / 2;
+    const long pair0 = (long)blockIdx.x * M;
     for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
         const int l = q / N, e = q % N;
-        const long row = row0 + l;
-        A[e * (M + 1) + l] = Cx<T>{row < rows ? src[row * N + e] : (T)0, (T)0};
+        const T* row = src + 2 * (pair0 + l) * N;
+        const bool ok = pair0 + l < pairs;
+        A[e * (M + 1) + l] = Cx<T>{ok ? row[e] : (T)0, ok ? row[N + e] : (T)0};
     }
     __syncthreads();
     Cx<T>* R = sstage<T, N, M, false, 0>(A, B, sw);
-    for (int q = threadIdx.x; q < M * nxh; q += blockDim.x) {
-        const int l = q / nxh, e = q % nxh;
-        const long row = row0 + l;
-        if (row < rows) C[row * nxh + e] = R[e * (M + 1) + l];
+    for (int q = threadIdx.x; q < M * nkeep; q += blockDim.x) {
+        const int l = q / nkeep, e = q % nkeep;
+        if (pair0 + l >= pairs) continue;
+        const Cx<T> u = R[e * (M + 1) + l], v = R[(e ? N - e : 0) * (M + 1) + l];
+        Cx<T>* dst = C + 2 * (pair0 + l) * pitch + e;
+        dst[0] = Cx<T>{(T)0.5 * (u.re + v.re), (T)0.5 * (u.im - v.im)};
+        dst[pitch] = Cx<T>{(T)0.5 * (u.im + v.im), (T)0.5 * (v.re - u.re)};
     }
 }
 
+// x pass, inverse, two real rows per complex line (Z = A + i B with A and B
+// extended by Hermitian symmetry; the imaginary parts of their zeroth and middle
+// coefficients, which no real row has, are dropped). Coefficients from nkeep on
+// are zero. Planes below *zsplit come from C2 (zsplit null: none does).
 template <typename T, int N, int M>
-__global__ void __launch_bounds__(256) ks_x_inv(Geo g, const T* tw, const Cx<T>* C, T* out) {
+__global__ void __launch_bounds__(256) ks_x_inv(Geo g, const T* tw, const Cx<T>* C, const Cx<T>* C2,
+                                                const int* zsplit, int nkeep, int pitch, T* out) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
-    constexpr int nxh = N / 2 + 1;
     Cx<T>* A = sw + N;
     Cx<T>* B = A + N * (M + 1);
     load_tw(sw, tw, N);
-    const long rows = (long)g.ny * g.nz;
-    const long row0 = (long)blockIdx.x * M;
-    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
-        const int l = q / N, e = q % N;
-        const long row = row0 + l;
-        Cx<T> v = {(T)0, (T)0};
-        if (row < rows) {
-            if (e < nxh) v = C[row * nxh + e];
-            else { v = C[row * nxh + (N - e)]; v.im = -v.im; }
+    const long pairs = (long)g.ny * g.nz / 2;
+    const long pair0 = (long)blockIdx.x * M;
+    const long low = zsplit ? (long)*zsplit * g.ny / 2 : 0;      // pairs of the planes below the split
+    for (int q = threadIdx.x; q < M * (N / 2 + 1); q += blockDim.x) {
+        const int l = q / (N / 2 + 1), e = q % (N / 2 + 1);
+        Cx<T> a = {(T)0, (T)0}, b = a;
+        if (pair0 + l < pairs && e < nkeep) {
+            const Cx<T>* row = (pair0 + l < low ? C2 : C) + 2 * (pair0 + l) * pitch + e;
+            a = row[0];
+            b = row[pitch];
         }
-        A[e * (M + 1) + l] = v;
+        if (e == 0 || e == N / 2) a.im = b.im = (T)0;
+        A[e * (M + 1) + l] = Cx<T>{a.re - b.im, a.im + b.re};
+        if (e > 0 && e < N / 2) A[(N - e) * (M + 1) + l] = Cx<T>{a.re + b.im, b.re - a.im};
     }
     __syncthreads();
     Cx<T>* R = sstage<T, N, M, true, 0>(A, B, sw);
     for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
         const int l = q / N, e = q % N;
-        const long row = row0 + l;
-        if (row < rows) out[row * N + e] = R[e * (M + 1) + l].re;
+        if (pair0 + l >= pairs) continue;
+        const Cx<T> v = R[e * (M + 1) + l];
+        T* row = out + 2 * (pair0 + l) * N;
+        row[e] = v.re;
+        row[N + e] = v.im;
     }
 }
 
@@ -492,7 +513,7 @@ void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>*
     const int nxh = g.nx / 2 + 1;
     const long rows = (long)g.ny * g.nz;
     switch (pass) {
-        case 0: ks_x_fwd<T, N, M><<<(int)((rows + M - 1) / M), 256, sm, s>>>(g, tw, src, C); break;
+        case 0: ks_x_fwd<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, src, C, nxh, nxh); break;
         case 1: ks_y<T, N, M, false><<<((nxh + M - 1) / M) * g.nz, 256, sm, s>>>(g, tw, C); break;
         case 2: {
             const T* l0 = sizeof(T) == 8 ? (const T*)p->lam[0] : (const T*)p->lam32[0];
@@ -502,7 +523,7 @@ void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>*
             break;
         }
         case 3: ks_y<T, N, M, true><<<((nxh + M - 1) / M) * g.nz, 256, sm, s>>>(g, tw, C); break;
-        case 4: ks_x_inv<T, N, M><<<(int)((rows + M - 1) / M), 256, sm, s>>>(g, tw, C, out); break;
+        case 4: ks_x_inv<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, C, nullptr, nullptr, nxh, nxh, out); break;
     }
 }
 
