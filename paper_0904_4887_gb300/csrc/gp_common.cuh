@@ -247,15 +247,53 @@ struct GammaTabs {
     int kt1;        // rows of exp(-n) a decaying term can use: floor(rcut) + 2
     int kg;         // rows of exp(+n) a growing term can use before it saturates
 };
+// The Eq. 9 sum split in two (k_gfar.cu): exp(-d) = near(d) + far(d), far(d) = exp(-d) w(d),
+// w(d) = erfc((d0 - d)/s)/2. near is summed over the images within rn on the grid, far
+// through its Fourier series with |k| <= K (smooth, so the series ends there).
+constexpr int kFarIv = 256, kFarDeg = 9;    // table of far's transform: intervals of |k| in [0, K], degree
+constexpr int kNearIv = 1024;               // tables of near(d) and -near'(d)/d: intervals of d^2 in [0, rn^2]
+constexpr int kNearDeg = 7, kNearSplit = 4; // their polynomials' degree; coefficients held as float pairs
+constexpr int kNearVec = 3;                 // float4 per interval: 4 pairs, 4 singles
+constexpr int kNearDirect = 16;             // intervals below this: near(d) by its formula (the square root's cusp)
+struct GammaFar {
+    double K, d0, s, rn, rcut;
+    int mx, my, mz;             // largest mode index per axis
+    double bx, by, bz;          // 2 pi / L
+    double inv_v;               // 1 / cell volume
+    double* ftab;               // [kFarIv][kFarDeg + 1]
+    float4 *ntab, *htab;        // [kNearIv][kNearVec]: near(d) and -near'(d)/d in t of each interval of d^2
+    float4 *ex, *ey, *ez;       // exp(i 2 pi m x_a / L) as two float pairs, [a][m + 1] per axis
+    float4* ezt;                // ez transposed, [m + 1][a]
+    double2 *s_all, *s_up;      // modes [2 mz + 1][2 my + 1][mx + 1]: every atom, kind 2: all but the lower layer
+    double2 *c_all, *c_up;      // [nz][ny][mx + 1] work arrays of the transforms
+    int* kz;                    // kind 2: kz[0] / kz[1] largest / smallest kzl of the lower atoms (0 / nz if none)
+    float2 idq, dq;             // 1/dq and dq as float pairs, dq = rn^2 / kNearIv
+    int k32;                    // intervals from k32 on are evaluated in FP32
+    float2 d0p, isp;            // d0 and 1/s as float pairs, for the direct branch
+    int up;                     // kind 2: the upper atoms have arrays of their own
+};
+size_t gamma_far_bytes(int n_atoms, const GammaFar& f, const Geo& g);
+void gamma_far_view(void* base, int n_atoms, GammaFar& f, const Geo& g);
+// tables of the split function alone (they depend on K, d0, s, rn and rcut)
+void launch_gamma_far_consts(const GammaFar& f, cudaStream_t s);
+// per-atom phases, then the modes of far's sum; kind 2: also those of the atoms above z_lim
+void launch_gamma_far_modes(const Geo& g, Atoms at, const GammaFar& f, const GAtom* ga, cudaStream_t s);
+// S_a += the far part of sum_i W_i d gamma_i / d R_a from the modes of W in s_all (and s_up)
+void launch_gamma_far_force(const Geo& g, int n_atoms, const GammaFar& f, const GAtom* ga, double* S, cudaStream_t s);
 size_t gamma_tabs_bytes(int n_atoms, int m, int nmax);
 GammaTabs gamma_tabs_view(void* base, int n_atoms, int m, int nmax);
 void launch_gamma_tables(const Geo& g, Atoms at, DielParams p, const double* rvdw, const GammaTabs& gt,
                          cudaStream_t s);
+// far (may be null): the split sum. gfar holds far's part of gamma at every point (build), or
+// receives W d eps/d gamma (force), pn the dielectric parameters with rn as the radius
 void launch_build_eps_gamma_df(const Geo& g, Atoms at, DielParams p, const GammaTabs& gt, double* eps64,
-                               double* fe64, float* eps32, cudaStream_t s);
+                               double* fe64, float* eps32, cudaStream_t s, const GammaFar* far = nullptr,
+                               const DielParams* pn = nullptr, const double* gfar = nullptr);
 // phid: phi as float pairs (read unless wext is given)
 void launch_forces_eps_gamma_df(const Geo& g, Atoms at, DielParams p, const GammaTabs& gt, const float2* phid,
-                                const double* wext, const double* fe64, double* S, cudaStream_t s);
+                                const double* wext, const double* fe64, double* S, cudaStream_t s,
+                                const GammaFar* far = nullptr, const DielParams* pn = nullptr,
+                                double* gfar = nullptr);
 // Periodized 1D Gaussian factor tables (k_fields.cu), Gaussian ge = 2 atom + {0 core, 1 cloud}
 struct GaussTabs {
     double* val;    // [G][3][nmax] X, Y, Z factors summed over the images -L, 0, +L
@@ -408,6 +446,11 @@ struct FFTPlan;
 FFTPlan* fft_create(const Geo& g, cudaStream_t s);
 void fft_destroy(FFTPlan* p);
 size_t fft_workspace_bytes(const Geo& g, bool dbl);
+// whether every extent has a compile-time transform (the band-limited transforms need them)
+bool fft_static_extents(const Geo& g);
+// band-limited transforms of the split Eq. 9 sum (FP64): modes -> grid field, and grid field -> modes
+void fft_band_inverse(FFTPlan* p, const GammaFar& f, double* out, cudaStream_t s);
+void fft_band_forward(FFTPlan* p, const GammaFar& f, const double* src, cudaStream_t s);
 // Solve L out = src (7-point Laplacian, periodic), k = 0 mode dropped.
 template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s);
 

@@ -15,6 +15,7 @@
 #include "gp_common.cuh"
 
 #include <algorithm>
+#include <iterator>
 #include <vector>
 
 namespace gp {
@@ -490,6 +491,92 @@ __global__ void __launch_bounds__(256) ks_z_solve(Geo g, const T* tw, const T* l
     }
 }
 
+// ---------------------------------------------------------------------------
+// Transforms of a band-limited periodic field (FP64; the Fourier part of the
+// Eq. 9 sum): modes |m_a| <= (f.mx, f.my, f.mz), stored [2 mz + 1][2 my + 1][mx + 1],
+// to and from the grid. A pass runs only the lines that can be nonzero: z on the
+// modes' (kx, ky) columns, y on the mx + 1 kept kx of every plane, x on all rows.
+template <int N, int M>
+__global__ void __launch_bounds__(256) kb_z_inv(const double* tw, int mx, int my, int mz, const Cx<double>* S,
+                                                Cx<double>* C, int ny) {
+    extern __shared__ unsigned char smem_raw[];
+    Cx<double>* sw = reinterpret_cast<Cx<double>*>(smem_raw);
+    Cx<double>* A = sw + N;
+    Cx<double>* B = A + N * (M + 1);
+    load_tw(sw, tw, N);
+    const int pitch = mx + 1, cols = 2 * my + 1, nchunks = (pitch + M - 1) / M;
+    const int kx0 = (blockIdx.x % nchunks) * M, jy = blockIdx.x / nchunks;      // ky = jy - my
+    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
+        const int e = q / M, l = q % M;
+        const int m = e <= mz ? e : e - N;                                      // kz of element e
+        Cx<double> v = {0.0, 0.0};
+        if (kx0 + l < pitch && m >= -mz) v = S[((long)(m + mz) * cols + jy) * pitch + kx0 + l];
+        A[e * (M + 1) + l] = v;
+    }
+    __syncthreads();
+    Cx<double>* R = sstage<double, N, M, true, 0>(A, B, sw);
+    const int j = jy >= my ? jy - my : jy - my + ny;
+    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
+        const int e = q / M, l = q % M;
+        if (kx0 + l < pitch) C[((long)e * ny + j) * pitch + kx0 + l] = R[e * (M + 1) + l];
+    }
+}
+
+// forward along z of the planes k0 <= k < k1 (the others taken as zero), the kept kz to the mode array
+template <int N, int M>
+__global__ void __launch_bounds__(256) kb_z_fwd(const double* tw, int mx, int my, int mz, const Cx<double>* C,
+                                                Cx<double>* S, int ny, const int* zsplit, int low) {
+    extern __shared__ unsigned char smem_raw[];
+    Cx<double>* sw = reinterpret_cast<Cx<double>*>(smem_raw);
+    Cx<double>* A = sw + N;
+    Cx<double>* B = A + N * (M + 1);
+    load_tw(sw, tw, N);
+    const int pitch = mx + 1, cols = 2 * my + 1, nchunks = (pitch + M - 1) / M;
+    const int kx0 = (blockIdx.x % nchunks) * M, jy = blockIdx.x / nchunks;
+    const int j = jy >= my ? jy - my : jy - my + ny;
+    const int zs = zsplit ? *zsplit : 0;
+    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
+        const int e = q / M, l = q % M;
+        Cx<double> v = {0.0, 0.0};
+        if (kx0 + l < pitch && (e < zs) == (low != 0)) v = C[((long)e * ny + j) * pitch + kx0 + l];
+        A[e * (M + 1) + l] = v;
+    }
+    __syncthreads();
+    Cx<double>* R = sstage<double, N, M, false, 0>(A, B, sw);
+    for (int q = threadIdx.x; q < M * (2 * mz + 1); q += blockDim.x) {
+        const int m = q / M - mz, l = q % M;
+        if (kx0 + l < pitch)
+            S[((long)(m + mz) * cols + jy) * pitch + kx0 + l] = R[(m < 0 ? m + N : m) * (M + 1) + l];
+    }
+}
+
+// along y in place, the mx + 1 kept kx of one plane. Inverse: ky beyond my are zero on
+// entry, planes below *zsplit are taken from C2; forward: only |ky| <= my is written.
+template <int N, int M, bool INV>
+__global__ void __launch_bounds__(256) kb_y(const double* tw, int mx, int my, Cx<double>* C, Cx<double>* C2,
+                                            const int* zsplit) {
+    extern __shared__ unsigned char smem_raw[];
+    Cx<double>* sw = reinterpret_cast<Cx<double>*>(smem_raw);
+    Cx<double>* A = sw + N;
+    Cx<double>* B = A + N * (M + 1);
+    load_tw(sw, tw, N);
+    const int pitch = mx + 1, nchunks = (pitch + M - 1) / M;
+    const int kx0 = (blockIdx.x % nchunks) * M;
+    const long k = blockIdx.x / nchunks;
+    Cx<double>* base = (zsplit && k < *zsplit ? C2 : C) + k * (long)pitch * N;
+    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
+        const int e = q / M, l = q % M;
+        const bool in = kx0 + l < pitch && (!INV || e <= my || e >= N - my);
+        A[e * (M + 1) + l] = in ? base[(long)e * pitch + kx0 + l] : Cx<double>{0.0, 0.0};
+    }
+    __syncthreads();
+    Cx<double>* R = sstage<double, N, M, INV, 0>(A, B, sw);
+    for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
+        const int e = q / M, l = q % M;
+        if (kx0 + l < pitch && (INV || e <= my || e >= N - my)) base[(long)e * pitch + kx0 + l] = R[e * (M + 1) + l];
+    }
+}
+
 template <typename T, int N>
 constexpr size_t smem_static() { return (size_t)N * sizeof(Cx<T>) * (1 + 2 * ((size_t)lines_static<T, N>() + 1)); }
 
@@ -524,6 +611,64 @@ void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>*
         }
         case 3: ks_y<T, N, M, true><<<((nxh + M - 1) / M) * g.nz, 256, sm, s>>>(g, tw, C); break;
         case 4: ks_x_inv<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, C, nullptr, nullptr, nxh, nxh, out); break;
+    }
+}
+
+// the band passes: 0 z inverse (up: of the upper atoms' modes), 1 y inverse, 2 x inverse, 3 x forward,
+// 4 y forward, 5 z forward (up: the planes below the split); f null sets the attributes only
+template <int N>
+void band_pass(int pass, FFTPlan* p, const GammaFar* f, bool up, const double* src, double* out, cudaStream_t s) {
+    constexpr int M = lines_static<double, N>();
+    constexpr size_t sm = smem_static<double, N>();
+    if (!f) {
+        const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        switch (pass) {
+            case 0: cudaFuncSetAttribute(kb_z_inv<N, M>, a, (int)sm); break;
+            case 1: cudaFuncSetAttribute(kb_y<N, M, true>, a, (int)sm); break;
+            case 4: cudaFuncSetAttribute(kb_y<N, M, false>, a, (int)sm); break;
+            case 5: cudaFuncSetAttribute(kb_z_fwd<N, M>, a, (int)sm); break;
+            default: break;                  // the x kernels are the vacuum solve's
+        }
+        return;
+    }
+    const Geo& g = p->g;
+    using C = Cx<double>;
+    const int pitch = f->mx + 1, nch = (pitch + M - 1) / M;
+    const int nx2 = (int)(((long)g.ny * g.nz / 2 + M - 1) / M);
+    C* ca = reinterpret_cast<C*>(f->c_all);
+    C* cu = reinterpret_cast<C*>(f->c_up);
+    C* sa = reinterpret_cast<C*>(f->s_all);
+    C* su = reinterpret_cast<C*>(f->s_up);
+    const int* zs = f->up ? f->kz : nullptr;
+    switch (pass) {
+        case 0: kb_z_inv<N, M><<<nch * (2 * f->my + 1), 256, sm, s>>>(p->tw64[2], f->mx, f->my, f->mz, up ? su : sa,
+                                                                      up ? cu : ca, g.ny); break;
+        case 1: kb_y<N, M, true><<<nch * g.nz, 256, sm, s>>>(p->tw64[1], f->mx, f->my, ca, cu, zs); break;
+        case 2: ks_x_inv<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], ca, cu, zs, pitch, pitch, out); break;
+        case 3: ks_x_fwd<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], src, ca, pitch, pitch); break;
+        case 4: kb_y<N, M, false><<<nch * g.nz, 256, sm, s>>>(p->tw64[1], f->mx, f->my, ca, cu, nullptr); break;
+        case 5: kb_z_fwd<N, M><<<nch * (2 * f->my + 1), 256, sm, s>>>(p->tw64[2], f->mx, f->my, f->mz, ca,
+                                                                      up ? su : sa, g.ny, zs, up ? 1 : 0); break;
+    }
+}
+
+bool dispatch_band(int n, int pass, FFTPlan* p, const GammaFar* f, bool up, const double* src, double* out,
+                   cudaStream_t s) {
+    switch (n) {
+        case 8: band_pass<8>(pass, p, f, up, src, out, s); return true;
+        case 12: band_pass<12>(pass, p, f, up, src, out, s); return true;
+        case 16: band_pass<16>(pass, p, f, up, src, out, s); return true;
+        case 24: band_pass<24>(pass, p, f, up, src, out, s); return true;
+        case 32: band_pass<32>(pass, p, f, up, src, out, s); return true;
+        case 48: band_pass<48>(pass, p, f, up, src, out, s); return true;
+        case 64: band_pass<64>(pass, p, f, up, src, out, s); return true;
+        case 96: band_pass<96>(pass, p, f, up, src, out, s); return true;
+        case 128: band_pass<128>(pass, p, f, up, src, out, s); return true;
+        case 192: band_pass<192>(pass, p, f, up, src, out, s); return true;
+        case 256: band_pass<256>(pass, p, f, up, src, out, s); return true;
+        case 384: band_pass<384>(pass, p, f, up, src, out, s); return true;
+        case 512: band_pass<512>(pass, p, f, up, src, out, s); return true;
+        default: return false;
     }
 }
 
@@ -616,6 +761,8 @@ FFTPlan* fft_create(const Geo& g, cudaStream_t s) {
     }
     set_fft_attributes<float>(g);
     set_fft_attributes<double>(g);
+    for (int pass : {0, 1, 4, 5}) dispatch_band(pass == 0 || pass == 5 ? g.nz : g.ny, pass, nullptr, nullptr, false,
+                                                nullptr, nullptr, nullptr);
     return p;
 }
 
@@ -632,6 +779,28 @@ void fft_destroy(FFTPlan* p) {
 
 size_t fft_workspace_bytes(const Geo& g, bool dbl) {
     return (size_t)(g.nx / 2 + 1) * g.ny * g.nz * 2 * (dbl ? sizeof(double) : sizeof(float));
+}
+
+bool fft_static_extents(const Geo& g) {
+    const int ns[] = {8, 12, 16, 24, 32, 48, 64, 96, 128, 192, 256, 384, 512};
+    auto has = [&](int n) { return std::find(std::begin(ns), std::end(ns), n) != std::end(ns); };
+    return has(g.nx) && has(g.ny) && has(g.nz);
+}
+
+void fft_band_inverse(FFTPlan* p, const GammaFar& f, double* out, cudaStream_t s) {
+    const Geo& g = p->g;
+    dispatch_band(g.nz, 0, p, &f, false, nullptr, nullptr, s);
+    if (f.up) dispatch_band(g.nz, 0, p, &f, true, nullptr, nullptr, s);
+    dispatch_band(g.ny, 1, p, &f, false, nullptr, nullptr, s);
+    dispatch_band(g.nx, 2, p, &f, false, nullptr, out, s);
+}
+
+void fft_band_forward(FFTPlan* p, const GammaFar& f, const double* src, cudaStream_t s) {
+    const Geo& g = p->g;
+    dispatch_band(g.nx, 3, p, &f, false, src, nullptr, s);
+    dispatch_band(g.ny, 4, p, &f, false, nullptr, nullptr, s);
+    dispatch_band(g.nz, 5, p, &f, false, nullptr, nullptr, s);
+    if (f.up) dispatch_band(g.nz, 5, p, &f, true, nullptr, nullptr, s);
 }
 
 template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s) {

@@ -9,6 +9,7 @@
 // keeps the survivors in shared memory, and then every thread runs over that
 // short list: in FP64, or in df64 (pairs of FP32 numbers) where a kernel says
 // so, because GB300's FP64 pipe runs at 1/64 of its FP32 rate.
+#include "df.cuh"
 #include "gp_common.cuh"
 
 namespace gp {
@@ -227,51 +228,6 @@ __global__ void __launch_bounds__(TT) k_build_eps(Geo g, Atoms at, DielParams p,
     }
 }
 
-// ----------------------------------------------------------------- df64
-// A value carried as an unevaluated sum hi + lo of two FP32 numbers (about 48
-// significant bits; Dekker 1971, Knuth's two-sum). The per-point sums of the
-// density and its force run in this form: a few FP32 instructions replace an
-// FP64 instruction that costs 64 FP32 issue slots on this GPU.
-struct df { float hi, lo; };
-
-__device__ __forceinline__ df df_from(double v) {
-    const float2 p = split_to_float2(v);      // the casts' result, without the FP64 pipe
-    return {p.x, p.y};
-}
-__device__ __forceinline__ double df_to(df a) { return f32_to_f64(a.hi) + f32_to_f64(a.lo); }
-__device__ __forceinline__ df as_df(float2 v) { return df{v.x, v.y}; }
-
-// (s, c): a compensated pair (value s + c) summed across the warp in place (Knuth two-sum per step)
-__device__ __forceinline__ void warp_sum_df(float& s, float& c) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-        const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
-        const float t = s + s2;
-        const float z = t - s;
-        c += c2 + ((s - (t - z)) + (s2 - z));
-        s = t;
-    }
-}
-
-__device__ __forceinline__ df df_quick(float s, float e) {   // |s| >= |e|
-    const float t = s + e;
-    return {t, e - (t - s)};
-}
-__device__ __forceinline__ df df_mul(df a, df b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    return df_quick(p, e);
-}
-__device__ __forceinline__ df df_add(df a, df b) {
-    const float s = a.hi + b.hi;
-    const float v = s - a.hi;
-    float e = (a.hi - (s - v)) + (b.hi - v);
-    e += a.lo + b.lo;
-    return df_quick(s, e);
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
@@ -349,19 +305,6 @@ __device__ __forceinline__ bool gauss_hits_tile(const GaussTabs& gt, int ge, con
     const int* w = gt.win + ge * 6;
     return span_hits(w[0], w[1], g.nx, t.i0, t.i1) && span_hits(w[2], w[3], g.ny, t.j0, t.j1) &&
            span_hits(w[4], w[5], g.nz, t.k0, t.k1);
-}
-
-// s += a * b with the product formed exactly to ~2^-48 (df64) and the sum
-// compensated (Neumaier): the FP32 pipe does the work of an FP64 FMA.
-__device__ __forceinline__ void df_acc(float& s, float& c, df a, df b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, e);
-    e = fmaf(a.lo, b.hi, e);
-    const float t = s + p;
-    const float z = t - s;
-    c += ((s - (t - z)) + (p - z)) + e;
-    s = t;
 }
 
 // ----------------------------------------------------------------- rho
@@ -1327,8 +1270,69 @@ __global__ void k_gamma_tables(Geo g, Atoms at, DielParams p, const double* rvdw
     }
 }
 
+// ----------------------------------------------------------------- the split sum's near part
+// near(d) = exp(-d) (1 - w(d)) (k_gfar.cu) of a pair from its squared distance x = d^2/dq in
+// table units, held as a float pair: interval (int)x, local variable t in [-1, 1], a degree-9
+// polynomial (Chebyshev; its first kNearSplit coefficients and its last steps in df).
+// The intervals below kNearDirect (d < rn/8), where the square root's branch point spoils
+// polynomials, take exp(-d) by its table and subtract far(d) < 2e-9, which FP32 gives.
+constexpr int kNearSmem = kNearIv * kNearVec * (int)sizeof(float4);
+__device__ __forceinline__ void near_table(float* dst, const float4* src) {
+    for (int q = threadIdx.x; q < kNearVec * kNearIv; q += blockDim.x) reinterpret_cast<float4*>(dst)[q] = __ldg(src + q);
+}
+
+// the polynomial of interval k at t in FP32 (leading floats only)
+__device__ __forceinline__ float near_poly32(const float* __restrict__ tab, int k, float t) {
+    const float4* r = reinterpret_cast<const float4*>(tab) + kNearVec * k;
+    const float4 a = r[0], b = r[1], c = r[2];          // h0 l0 h1 l1 | h2 l2 h3 l3 | 4 5 6 7
+    float v = fmaf(c.w, t, c.z);
+    v = fmaf(v, t, c.y);
+    v = fmaf(v, t, c.x);
+    v = fmaf(v, t, b.z);
+    v = fmaf(v, t, b.x);
+    v = fmaf(v, t, a.z);
+    return fmaf(v, t, a.x);
+}
+
+__device__ __forceinline__ df near_poly(const float* __restrict__ tab, int k, df t) {
+    const float4* r = reinterpret_cast<const float4*>(tab) + kNearVec * k;
+    const float4 a = r[0], b = r[1], c = r[2];
+    float v = fmaf(c.w, t.hi, c.z);
+    v = fmaf(v, t.hi, c.y);
+    v = fmaf(v, t.hi, c.x);
+    df acc = df_horner(df{v, 0.f}, t, b.z, b.w);
+    acc = df_horner(acc, t, b.x, b.y);
+    acc = df_horner(acc, t, a.z, a.w);
+    return df_horner(acc, t, a.x, a.y);
+}
+
+// w(d) and w'(d) of a pair in the direct branch, where w < 2e-9: FP32, with u = (d0 - d)/s as a
+// float pair (the argument's own rounding would move w by 2e-6 of it, all pairs the same way)
+__device__ __forceinline__ float2 near_window(const GammaFar& gf, df d) {
+    const float a = gf.d0p.x - d.hi;
+    const float bb = a - gf.d0p.x;
+    const float al = (gf.d0p.x - (a - bb)) - (d.hi + bb) + (gf.d0p.y - d.lo);
+    const float u = a * gf.isp.x;
+    const float ul = fmaf(a, gf.isp.x, -u) + fmaf(a, gf.isp.y, al * gf.isp.x);
+    const float u2 = u * u;
+    const float e = expf(-u2) * (1.f - (fmaf(u, u, -u2) + 2.f * u * ul)) * 0.56418958f;   // exp(-u^2)/sqrt(pi)
+    return make_float2(fmaf(-e, ul, 0.5f * erfcf(u)), e * gf.isp.x);
+}
+
+// t = 2 (x - k) - 1 as a float pair (x - k is exact in the leading float)
+__device__ __forceinline__ df near_local(df x, int k) {
+    const float a = 2.f * (x.hi - (float)k);
+    const float s = a - 1.f;
+    const float bb = s - a;
+    const float e = (a - (s - bb)) + (-1.f - bb) + 2.f * x.lo;
+    return df_quick(s, e);
+}
+
+template <bool kFar>
 __global__ void __launch_bounds__(TT, 2) k_build_eps_gamma_df(Geo g, Atoms at, DielParams p, GammaTabs gt,
-                                                           double* eps64, double* fe64, float* eps32) {
+                                                           double* eps64, double* fe64, float* eps32,
+                                                           DielParams pn, GammaFar gf, const double* gfar) {
+    extern __shared__ __align__(16) float ntab[];      // kFar: near(d), kNearIv rows of kNearVec float4
     __shared__ int elist[GCAP];
     __shared__ df sx2[GB][TX];
     __shared__ df sy2[GB][TY];
@@ -1409,71 +1413,162 @@ __global__ void __launch_bounds__(TT, 2) k_build_eps_gamma_df(Geo g, Atoms at, D
             }
         }
     }
-    // the decaying terms over every atom image within rcut
     for (int q = threadIdx.x; q < 256; q += TT) stab[q] = as_df(__ldg(gt.t2 + q));
-    const int nxi = 2 * p.mx + 1, nyi = 2 * p.my + 1, nimg = nxi * nyi * (2 * p.mz + 1);
-    const int nq = at.n * nimg;
-    const float reach = p.rcutf + kMargin, rc2f = p.rc2f, far2f = p.far2f;
-    auto keep = [&](int q) {
-        float fx, fy, fz;
-        gimage32(at.w32, q / nimg, q % nimg, g, p, fx, fy, fz);
-        return box_d2(t, fx, fy, fz) < reach * reach;
-    };
-    const int total = block_compact(0, nq, keep, nullptr, scratch);
-    const int win = total <= GCAP ? nq : GCAP;       // GCAP candidates never overflow the list
-    const int ns = NS + gt.kt1;
-    for (int w0 = 0; w0 < nq; w0 += win) {
-        const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
-        for (int e0 = 0; e0 < m; e0 += GB) {
-            const int ms = min(GB, m - e0);
-            for (int r = threadIdx.x; r < ms * ns; r += TT) {
-                const int e = r / ns, c = r % ns;
-                const int q = elist[e0 + e];
-                const int a = q / nimg, im = q % nimg;
-                if (c < NS) {
-                    int axis, gi;
-                    staged_line(t, g, c, axis, gi);
-                    const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(p, im, axis), axis, gi)));
-                    const df sq = df_mul(dd, dd);
-                    if (c < TX) sx2[e][c] = sq;
-                    else if (c < TX + TY) sy2[e][c - TX] = sq;
-                    else sz2[e][c - TX - TY] = sq;
-                } else {
-                    const int n = c - NS;
-                    srow[e][n] = df_mul(as_df(gt.at[a].a), as_df(__ldg(gt.t1 + n)));
-                    if (n == 0) {
-                        skz[e] = eq19 ? gt.at[a].kzl : 0;
-                        sqs[e] = gt.at[a].l2a;
+    // kind 2 with the split sum: planes from kzs on take every atom's far part from gfar, planes
+    // below it only the upper atoms'; a lower atom's planes kz .. kzs - 1 sum its whole term
+    int kzs = 0;
+    if constexpr (kFar) {
+        kzs = gf.up ? gf.kz[0] : 0;
+        near_table(ntab, gf.ntab);
+        const int nxi = 2 * pn.mx + 1, nyi = 2 * pn.my + 1, nimg = nxi * nyi * (2 * pn.mz + 1);
+        const int nq = at.n * nimg;
+        const float reach = pn.rcutf + kMargin, xend = (float)kNearIv;
+        const df idq = as_df(gf.idq), dq = as_df(gf.dq);
+        auto keep = [&](int q) {
+            float fx, fy, fz;
+            gimage32(at.w32, q / nimg, q % nimg, g, pn, fx, fy, fz);
+            return box_d2(t, fx, fy, fz) < reach * reach;
+        };
+        const int total = block_compact(0, nq, keep, nullptr, scratch);
+        const int win = total <= GCAP ? nq : GCAP;
+        constexpr int nrow = 4, ns = NS + nrow;          // the direct branch has d < 3
+        for (int w0 = 0; w0 < nq; w0 += win) {
+            const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
+            for (int e0 = 0; e0 < m; e0 += GB) {
+                const int ms = min(GB, m - e0);
+                for (int r = threadIdx.x; r < ms * ns; r += TT) {
+                    const int e = r / ns, c = r % ns;
+                    const int q = elist[e0 + e];
+                    const int a = q / nimg, im = q % nimg;
+                    if (c < NS) {
+                        int axis, gi;
+                        staged_line(t, g, c, axis, gi);
+                        const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(pn, im, axis), axis, gi)));
+                        const df sq = df_mul(df_mul(dd, dd), idq);
+                        if (c < TX) sx2[e][c] = sq;
+                        else if (c < TX + TY) sy2[e][c - TX] = sq;
+                        else sz2[e][c - TX - TY] = sq;
+                    } else {
+                        // rows 0 .. 3: exp(rvdw - n); row 0 alone scales the table's terms
+                        const int n = c - NS;
+                        srow[e][n] = df_mul(as_df(gt.at[a].a), as_df(__ldg(gt.t1 + n)));
+                        if (n == 0) skz[e] = gf.up && gt.at[a].kzl > 0 ? kzs : 0;
                     }
                 }
-            }
-            __syncthreads();
-            for (int e = 0; e < ms; ++e) {
-                const df xy = df_add(sx2[e][tx], sy2[e][ty]);
-                if (!(xy.hi < rc2f)) continue;                      // beyond rcut for every plane
-                const int kz = skz[e];                              // below a lower atom: its growing term instead
-                const float l2a = sqs[e];
+                __syncthreads();
+                for (int e = 0; e < ms; ++e) {
+                    const df xy = df_add(sx2[e][tx], sy2[e][ty]);
+                    if (!(xy.hi < xend)) continue;
+                    const int kz = skz[e];
+                    const df A = srow[e][0];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int zz = tz + 4 * r;
+                        const float xf = xy.hi + sz2[e][zz].hi;
+                        if (!(xf < xend) || !valid[r] || sat[r] || t.k0 + zz < kz) continue;
+                        if ((int)xf >= gf.k32) {
+                            const int k = (int)xf;
+                            const float v = near_poly32(ntab, k, fmaf(2.f, xf - (float)k, -1.f));
+                            df_add_to(F[r], G[r], df{A.hi * v, 0.f});
+                            continue;
+                        }
+                        const df x = df_add(xy, sz2[e][zz]);
+                        const int k = (int)x.hi;
+                        df v;
+                        if (k >= kNearDirect) {
+                            v = df_mul(near_poly(ntab, k, near_local(x, k)), A);
+                        } else {
+                            const df q = df_mul(x, dq);
+                            float y;
+                            int n;
+                            const df d = q.hi > 0.f ? df_sqrt(q, y) : df{0.f, 0.f};
+                            v = exp_tab<true>(d, srow[e], stab, n);
+                            v = df_add(v, df{-A.hi * expf(-d.hi) * near_window(gf, d).x, 0.f});
+                        }
+                        df_add_to(F[r], G[r], v);
+                    }
+                }
+                // the batch's df sums into FP64: a df sum loses half a unit of 2^-48 of itself per
+                // term, so it is kept short (one for all the images lost 5e-14 of eps; the casts and
+                // adds run on the FP64 pipe beside the other warps' FP32 work)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const int zz = tz + 4 * r;
-                    if (!valid[r] || sat[r] || t.k0 + zz < kz) continue;
-                    const float qf = xy.hi + sz2[e][zz].hi;
-                    if (qf >= far2f) {
-                        if (!(qf < rc2f)) continue;
-                        float y;
-                        df_add_to(F[r], G[r], df{exp_far(sqrt_f32(qf, y), l2a), 0.f});
-                        continue;
-                    }
-                    const df q = df_add(xy, sz2[e][zz]);
-                    if (!(q.hi < rc2f)) continue;
-                    float y;
-                    int n;
-                    const df d = q.hi > 0.f ? df_sqrt(q, y) : df{0.f, 0.f};
-                    const df v = exp_tab<true>(d, srow[e], stab, n);
-                    gamma_acc(D[r], F[r], G[r], v, n);
+                    D[r] += (double)F[r] + (double)G[r];
+                    F[r] = G[r] = 0.f;
                 }
+                __syncthreads();
             }
-            __syncthreads();
+        }
+    }
+    // the decaying terms over every atom image within rcut (with the split sum: the lower atoms' at
+    // the planes between the lowest and the highest of them)
+    if (!kFar || (gf.up && t.k0 < kzs && t.k1 >= gf.kz[1])) {
+        const int nxi = 2 * p.mx + 1, nyi = 2 * p.my + 1, nimg = nxi * nyi * (2 * p.mz + 1);
+        const int nq = at.n * nimg;
+        const int kend = kFar ? kzs : g.nz;
+        const float reach = p.rcutf + kMargin, rc2f = p.rc2f, far2f = p.far2f;
+        auto keep = [&](int q) {
+            if (kFar && gt.at[q / nimg].kzl <= 0) return false;
+            float fx, fy, fz;
+            gimage32(at.w32, q / nimg, q % nimg, g, p, fx, fy, fz);
+            return box_d2(t, fx, fy, fz) < reach * reach;
+        };
+        const int total = block_compact(0, nq, keep, nullptr, scratch);
+        const int win = total <= GCAP ? nq : GCAP;       // GCAP candidates never overflow the list
+        const int ns = NS + gt.kt1;
+        for (int w0 = 0; w0 < nq; w0 += win) {
+            const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
+            for (int e0 = 0; e0 < m; e0 += GB) {
+                const int ms = min(GB, m - e0);
+                for (int r = threadIdx.x; r < ms * ns; r += TT) {
+                    const int e = r / ns, c = r % ns;
+                    const int q = elist[e0 + e];
+                    const int a = q / nimg, im = q % nimg;
+                    if (c < NS) {
+                        int axis, gi;
+                        staged_line(t, g, c, axis, gi);
+                        const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(p, im, axis), axis, gi)));
+                        const df sq = df_mul(dd, dd);
+                        if (c < TX) sx2[e][c] = sq;
+                        else if (c < TX + TY) sy2[e][c - TX] = sq;
+                        else sz2[e][c - TX - TY] = sq;
+                    } else {
+                        const int n = c - NS;
+                        srow[e][n] = df_mul(as_df(gt.at[a].a), as_df(__ldg(gt.t1 + n)));
+                        if (n == 0) {
+                            skz[e] = eq19 ? gt.at[a].kzl : 0;
+                            sqs[e] = gt.at[a].l2a;
+                        }
+                    }
+                }
+                __syncthreads();
+                for (int e = 0; e < ms; ++e) {
+                    const df xy = df_add(sx2[e][tx], sy2[e][ty]);
+                    if (!(xy.hi < rc2f)) continue;                      // beyond rcut for every plane
+                    const int kz = skz[e];                              // below a lower atom: its growing term instead
+                    const float l2a = sqs[e];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int zz = tz + 4 * r;
+                        if (!valid[r] || sat[r] || t.k0 + zz < kz || (kFar && t.k0 + zz >= kend)) continue;
+                        const float qf = xy.hi + sz2[e][zz].hi;
+                        if (qf >= far2f) {
+                            if (!(qf < rc2f)) continue;
+                            float y;
+                            df_add_to(F[r], G[r], df{exp_far(sqrt_f32(qf, y), l2a), 0.f});
+                            continue;
+                        }
+                        const df q = df_add(xy, sz2[e][zz]);
+                        if (!(q.hi < rc2f)) continue;
+                        float y;
+                        int n;
+                        const df d = q.hi > 0.f ? df_sqrt(q, y) : df{0.f, 0.f};
+                        const df v = exp_tab<true>(d, srow[e], stab, n);
+                        gamma_acc(D[r], F[r], G[r], v, n);
+                    }
+                }
+                __syncthreads();
+            }
         }
     }
 #pragma unroll
@@ -1484,7 +1579,8 @@ __global__ void __launch_bounds__(TT, 2) k_build_eps_gamma_df(Geo g, Atoms at, D
         if (sat[r]) {
             e = 1.0;
         } else {
-            const double gam = D[r] + (f32_to_f64(F[r]) + f32_to_f64(G[r]));
+            double gam = D[r] + (f32_to_f64(F[r]) + f32_to_f64(G[r]));
+            if constexpr (kFar) gam += gfar[idx];
             if (gam > 0.0) {
                 const double gb = exp(p.beta2 * log(gam));         // gamma^(2 beta)
                 const double den = 1.0 + gb;
@@ -1507,9 +1603,12 @@ constexpr float kFarF2 = 18.f * 18.f;
 // order, so each atom's images are adjacent; every warp takes a contiguous share of
 // it, one image at a time over the tile's 2048 points (compensated FP32 sums of df
 // products), and turns its sums into FP64 atomics only when the atom changes.
+template <bool kFar>
 __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, DielParams p, GammaTabs gt,
                                                             const float2* phid, const double* wext,
-                                                            const double* fe64, double* S) {
+                                                            const double* fe64, double* S, DielParams pn,
+                                                            GammaFar gf, double* gfar) {
+    extern __shared__ __align__(16) float ntab[];      // kFar: -near'(d)/d, kNearIv rows of kNearVec float4
     __shared__ df Ws[TX * TY * EZ];              // W (d eps/d gamma), index tx + TX (ty + TY z)
     __shared__ int elist[GCAPF];
     __shared__ df wd[TT / 32][NS];               // a warp's image: displacements of the staged lines
@@ -1531,6 +1630,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
                 const long c = i + (long)g.nx * (j + (long)g.ny * k);
                 const df nw = neg_force_weight_df(g, phid, wext, fe64[c], i, j, k, c, c2x, c2y, c2z);
                 w = df{-nw.hi, -nw.lo};
+                if constexpr (kFar) gfar[c] = df_to(w);       // for the far part's transform
             }
             Ws[q] = w;
             any |= w.hi != 0.f;
@@ -1557,7 +1657,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
     // one image (displacements in wd, squares in wq, factor row in wrow) over the
     // tile's points: a decaying term at the planes k >= kz within rcut, a growing
     // term (grow) at the planes k < kz
-    auto pairs = [&](int kz, bool grow) {
+    auto pairs = [&](int kz, bool grow, int kend) {
         for (int b = 0; b < 16; ++b) {
             int tx, ty, tz;
             compact_point(b, lane, tx, ty, tz);
@@ -1568,7 +1668,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
             for (int r = 0; r < 4; ++r) {
                 const int zz = tz + 4 * r;
                 const int k = t.k0 + zz;
-                if (k >= g.nz || (grow ? k >= kz : k < kz)) continue;
+                if (k >= kend || (grow ? k >= kz : k < kz)) continue;
                 const df W = Ws[tx + TX * (ty + TY * zz)];
                 if (W.hi == 0.f) continue;                          // also every saturated point
                 if (!grow) {
@@ -1601,45 +1701,136 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
             }
         }
     };
-    // decaying terms
-    for (int q = threadIdx.x; q < 256; q += TT) stab[q] = as_df(__ldg(gt.t2 + q));
-    const int nxi = 2 * p.mx + 1, nyi = 2 * p.my + 1, nimg = nxi * nyi * (2 * p.mz + 1);
-    const int nq = at.n * nimg;
-    const float reach = p.rcutf + kMargin;
-    auto keep = [&](int q) {
-        float fx, fy, fz;
-        gimage32(at.w32, q / nimg, q % nimg, g, p, fx, fy, fz);
-        return box_d2(t, fx, fy, fz) < reach * reach;
-    };
-    const int total = block_compact(0, nq, keep, nullptr, scratch);
-    const int win = total <= GCAPF ? nq : GCAPF;
-    for (int w0 = 0; w0 < nq; w0 += win) {
-        const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
-        const int e1 = (int)(((long)(warp + 1) * m) / (TT / 32));
-        int cur = -1;
-        for (int e = (int)(((long)warp * m) / (TT / 32)); e < e1; ++e) {
-            const int q = elist[e];
-            const int a = q / nimg, im = q % nimg;
-            if (a != cur) {
-                if (cur >= 0) flush(cur);
-                cur = a;
+    // the split sum's near part of one image (squares in wq in table units)
+    auto near_pairs = [&](int kz, df A, df dq) {
+        for (int b = 0; b < 16; ++b) {
+            int tx, ty, tz;
+            compact_point(b, lane, tx, ty, tz);
+            if (t.i0 + tx >= g.nx || t.j0 + ty >= g.ny) continue;
+            const df xy = df_add(wq[warp][tx], wq[warp][TX + ty]);
+            if (!(xy.hi < (float)kNearIv)) continue;
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int zz = tz + 4 * r;
+                const int k = t.k0 + zz;
+                const float xf = xy.hi + wq[warp][TX + TY + zz].hi;
+                if (!(xf < (float)kNearIv) || k >= g.nz || k < kz) continue;
+                const df W = Ws[tx + TX * (ty + TY * zz)];
+                if (W.hi == 0.f) continue;
+                if ((int)xf >= gf.k32) {
+                    const int iv = (int)xf;
+                    const float c = W.hi * A.hi * near_poly32(ntab, iv, fmaf(2.f, xf - (float)iv, -1.f));
+                    fx = fmaf(c, wd[warp][tx].hi, fx);
+                    fy = fmaf(c, wd[warp][TX + ty].hi, fy);
+                    fz = fmaf(c, wd[warp][TX + TY + zz].hi, fz);
+                    continue;
+                }
+                const df x = df_add(xy, wq[warp][TX + TY + zz]);
+                const int iv = (int)x.hi;
+                df c;
+                if (iv >= kNearDirect) {
+                    c = df_mul(df_mul(near_poly(ntab, iv, near_local(x, iv)), A), W);
+                } else {
+                    const df q = df_mul(x, dq);
+                    if (!(q.hi > 0.f)) continue;
+                    float y;
+                    const df d = df_sqrt(q, y);
+                    int n;
+                    const float2 w = near_window(gf, d);             // -near' = exp(-d) (1 - w + w')
+                    c = df_add(exp_tab<true>(d, wrow[warp], stab, n), df{A.hi * expf(-d.hi) * (w.y - w.x), 0.f});
+                    c = df_mul(df_mul(W, c), df_recip(d, y));
+                }
+                df_acc(sx, cx, c, wd[warp][tx]);
+                df_acc(sy, cy, c, wd[warp][TX + ty]);
+                df_acc(sz, cz, c, wd[warp][TX + TY + zz]);
             }
-            __syncwarp();
-            for (int c = lane; c < NS; c += 32) {
-                int axis, gi;
-                staged_line(t, g, c, axis, gi);
-                const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(p, im, axis), axis, gi)));
-                wd[warp][c] = dd;
-                wq[warp][c] = df_mul(dd, dd);
-            }
-            const df A = as_df(gt.at[a].a);
-            l2a = gt.at[a].l2a;
-            for (int n = lane; n < gt.kt1; n += 32) wrow[warp][n] = df_mul(A, as_df(__ldg(gt.t1 + n)));
-            __syncwarp();
-            pairs(eq19 ? gt.at[a].kzl : 0, false);
         }
-        if (cur >= 0) flush(cur);
-        __syncthreads();                          // the list is read; the next window rebuilds it
+    };
+    for (int q = threadIdx.x; q < 256; q += TT) stab[q] = as_df(__ldg(gt.t2 + q));
+    int kzs = 0;                                  // kind 2 with the split sum: as in the build
+    if constexpr (kFar) {
+        kzs = gf.up ? gf.kz[0] : 0;
+        near_table(ntab, gf.htab);
+        const int nxi = 2 * pn.mx + 1, nyi = 2 * pn.my + 1, nimg = nxi * nyi * (2 * pn.mz + 1);
+        const int nq = at.n * nimg;
+        const float reach = pn.rcutf + kMargin;
+        const df idq = as_df(gf.idq), dq = as_df(gf.dq);
+        auto keep = [&](int q) {
+            float cx_, cy_, cz_;
+            gimage32(at.w32, q / nimg, q % nimg, g, pn, cx_, cy_, cz_);
+            return box_d2(t, cx_, cy_, cz_) < reach * reach;
+        };
+        const int total = block_compact(0, nq, keep, nullptr, scratch);
+        const int win = total <= GCAPF ? nq : GCAPF;
+        for (int w0 = 0; w0 < nq; w0 += win) {
+            const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
+            const int e1 = (int)(((long)(warp + 1) * m) / (TT / 32));
+            int cur = -1;
+            for (int e = (int)(((long)warp * m) / (TT / 32)); e < e1; ++e) {
+                const int q = elist[e];
+                const int a = q / nimg, im = q % nimg;
+                if (a != cur) {
+                    if (cur >= 0) flush(cur);
+                    cur = a;
+                }
+                __syncwarp();
+                for (int c = lane; c < NS; c += 32) {
+                    int axis, gi;
+                    staged_line(t, g, c, axis, gi);
+                    const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(pn, im, axis), axis, gi)));
+                    wd[warp][c] = dd;
+                    wq[warp][c] = df_mul(df_mul(dd, dd), idq);
+                }
+                const df A = as_df(gt.at[a].a);
+                if (lane < 4) wrow[warp][lane] = df_mul(A, as_df(__ldg(gt.t1 + lane)));
+                __syncwarp();
+                near_pairs(gf.up && gt.at[a].kzl > 0 ? kzs : 0, A, dq);
+            }
+            if (cur >= 0) flush(cur);
+            __syncthreads();                      // the list is read; the next window rebuilds it
+        }
+    }
+    // decaying terms (with the split sum: the lower atoms' at the planes between them)
+    if (!kFar || (gf.up && t.k0 < kzs && t.k1 >= gf.kz[1])) {
+        const int nxi = 2 * p.mx + 1, nyi = 2 * p.my + 1, nimg = nxi * nyi * (2 * p.mz + 1);
+        const int nq = at.n * nimg;
+        const float reach = p.rcutf + kMargin;
+        auto keep = [&](int q) {
+            if (kFar && gt.at[q / nimg].kzl <= 0) return false;
+            float cx_, cy_, cz_;
+            gimage32(at.w32, q / nimg, q % nimg, g, p, cx_, cy_, cz_);
+            return box_d2(t, cx_, cy_, cz_) < reach * reach;
+        };
+        const int total = block_compact(0, nq, keep, nullptr, scratch);
+        const int win = total <= GCAPF ? nq : GCAPF;
+        for (int w0 = 0; w0 < nq; w0 += win) {
+            const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
+            const int e1 = (int)(((long)(warp + 1) * m) / (TT / 32));
+            int cur = -1;
+            for (int e = (int)(((long)warp * m) / (TT / 32)); e < e1; ++e) {
+                const int q = elist[e];
+                const int a = q / nimg, im = q % nimg;
+                if (a != cur) {
+                    if (cur >= 0) flush(cur);
+                    cur = a;
+                }
+                __syncwarp();
+                for (int c = lane; c < NS; c += 32) {
+                    int axis, gi;
+                    staged_line(t, g, c, axis, gi);
+                    const df dd = as_df(__ldg(gt.d + gtab_index(gt, a, image_digit(p, im, axis), axis, gi)));
+                    wd[warp][c] = dd;
+                    wq[warp][c] = df_mul(dd, dd);
+                }
+                const df A = as_df(gt.at[a].a);
+                l2a = gt.at[a].l2a;
+                for (int n = lane; n < gt.kt1; n += 32) wrow[warp][n] = df_mul(A, as_df(__ldg(gt.t1 + n)));
+                __syncwarp();
+                pairs(eq19 ? gt.at[a].kzl : 0, false, kFar ? min(kzs, g.nz) : g.nz);
+            }
+            if (cur >= 0) flush(cur);
+            __syncthreads();                      // the list is read; the next window rebuilds it
+        }
     }
     if (!eq19) return;
     // growing terms: each lower atom's nearest image at the points below it
@@ -1661,7 +1852,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
             const df B = as_df(gt.at[a].b);
             for (int n = lane; n < gt.kg; n += 32) wrow[warp][n] = df_mul(B, as_df(__ldg(gt.u1 + n)));
             __syncwarp();
-            pairs(gt.at[a].kzl, true);
+            pairs(gt.at[a].kzl, true, g.nz);
             flush(a);
         }
         __syncthreads();                          // the list is read; the next window rebuilds it
@@ -2041,13 +2232,29 @@ void launch_gamma_tables(const Geo& g, Atoms at, DielParams p, const double* rvd
 }
 
 void launch_build_eps_gamma_df(const Geo& g, Atoms at, DielParams p, const GammaTabs& gt, double* eps64,
-                               double* fe64, float* eps32, cudaStream_t s) {
-    k_build_eps_gamma_df<<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, gt, eps64, fe64, eps32);
+                               double* fe64, float* eps32, cudaStream_t s, const GammaFar* far, const DielParams* pn,
+                               const double* gfar) {
+    if (!far) {
+        k_build_eps_gamma_df<false><<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, gt, eps64, fe64, eps32, p, GammaFar{},
+                                                                   nullptr);
+        return;
+    }
+    // the attribute belongs to the device: set on every call rather than remembered per process
+    cudaFuncSetAttribute(k_build_eps_gamma_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmem);
+    k_build_eps_gamma_df<true><<<tile_grid_ez(g), TT, kNearSmem, s>>>(g, at, p, gt, eps64, fe64, eps32, *pn, *far, gfar);
 }
 
 void launch_forces_eps_gamma_df(const Geo& g, Atoms at, DielParams p, const GammaTabs& gt, const float2* phid,
-                                const double* wext, const double* fe64, double* S, cudaStream_t s) {
-    k_forces_eps_gamma_df<<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, gt, phid, wext, fe64, S);
+                                const double* wext, const double* fe64, double* S, cudaStream_t s,
+                                const GammaFar* far, const DielParams* pn, double* gfar) {
+    if (!far) {
+        k_forces_eps_gamma_df<false><<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, gt, phid, wext, fe64, S, p, GammaFar{},
+                                                                    nullptr);
+        return;
+    }
+    cudaFuncSetAttribute(k_forces_eps_gamma_df<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNearSmem);
+    k_forces_eps_gamma_df<true><<<tile_grid_ez(g), TT, kNearSmem, s>>>(g, at, p, gt, phid, wext, fe64, S, *pn, *far,
+                                                                       gfar);
 }
 
 void launch_plane_max(const Geo& g, const double* eps64, double* out, cudaStream_t s) {
