@@ -423,6 +423,7 @@ template <typename T> void launch_coarse_vcycle(const CoarseSet<T>& S, cudaStrea
 void coarse_vcycle_init();    // allow the shared-memory variant its dynamic shared memory (before any capture)
 
 // dry/wet band (k_mg.cu)
+template <typename T> void launch_rsqrt(long n, const T* src, T* dst, cudaStream_t s);
 template <typename T> void launch_cast_eps(long n, const double* e64, T* eT, cudaStream_t s);
 template <typename T> void launch_band_eps(const Geo& g, const T* epsT, int first_interior, int band_nz,
                                            T* band_eps, cudaStream_t s);
@@ -451,7 +452,9 @@ bool fft_static_extents(const Geo& g);
 // band-limited transforms of the split Eq. 9 sum (FP64): modes -> grid field, and grid field -> modes
 void fft_band_inverse(FFTPlan* p, const GammaFar& f, double* out, cudaStream_t s);
 void fft_band_forward(FFTPlan* p, const GammaFar& f, const double* src, cudaStream_t s);
-// Solve L out = src (7-point Laplacian, periodic), k = 0 mode dropped.
-template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s);
+// Solve L out = src (7-point Laplacian, periodic), k = 0 mode dropped; with a field sc, out =
+// sc L^-1 (sc src) point by point.
+template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s,
+                                       const T* sc = nullptr);
 
 }  // namespace gp

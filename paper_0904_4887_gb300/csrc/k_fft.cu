@@ -136,7 +136,7 @@ __device__ void load_tw(Cx<T>* s, const T* tw, int n) {
 
 // x pass, forward: rows (j,k) of real input -> half spectrum
 template <typename T>
-__global__ void k_fft_x_fwd(Geo g, AxisPlan ap, const T* tw, int M, const T* src, Cx<T>* C) {
+__global__ void k_fft_x_fwd(Geo g, AxisPlan ap, const T* tw, int M, const T* src, const T* sc, Cx<T>* C) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
     const int N = g.nx, nxh = g.nx / 2 + 1;
@@ -148,7 +148,9 @@ __global__ void k_fft_x_fwd(Geo g, AxisPlan ap, const T* tw, int M, const T* src
     for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
         const int l = q / N, e = q % N;
         const long row = row0 + l;
-        A[e * M + l] = Cx<T>{row < rows ? src[row * N + e] : (T)0, (T)0};
+        T v = row < rows ? src[row * N + e] : (T)0;
+        if (sc && row < rows) v *= sc[row * N + e];
+        A[e * M + l] = Cx<T>{v, (T)0};
     }
     __syncthreads();
     Cx<T>* R = smem_fft<T, false>(A, B, N, M, ap, sw);
@@ -161,7 +163,7 @@ __global__ void k_fft_x_fwd(Geo g, AxisPlan ap, const T* tw, int M, const T* src
 
 // x pass, inverse: half spectrum rows -> real output (real part of the full line)
 template <typename T>
-__global__ void k_fft_x_inv(Geo g, AxisPlan ap, const T* tw, int M, const Cx<T>* C, T* out) {
+__global__ void k_fft_x_inv(Geo g, AxisPlan ap, const T* tw, int M, const Cx<T>* C, const T* sc, T* out) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
     const int N = g.nx, nxh = g.nx / 2 + 1;
@@ -185,7 +187,7 @@ __global__ void k_fft_x_inv(Geo g, AxisPlan ap, const T* tw, int M, const Cx<T>*
     for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
         const int l = q / N, e = q % N;
         const long row = row0 + l;
-        if (row < rows) out[row * N + e] = R[e * M + l].re;
+        if (row < rows) out[row * N + e] = R[e * M + l].re * (sc ? sc[row * N + e] : (T)1);
     }
 }
 
@@ -355,9 +357,11 @@ constexpr int lines_static() {
 // 192 x 192 x 384 FP64 solve took 3.15 ms with one row per line, 2.56 ms with two;
 // 128 x 128 x 256 in FP32 0.137 and 0.125 ms). The rows of a pair are neighbours
 // (ny is even for every extent the library takes).
-// The first nkeep coefficients of each row go to C, rows `pitch` apart.
+// The first nkeep coefficients of each row go to C, rows `pitch` apart. The source is
+// multiplied by sc point by point on the way in (sc null: not).
 template <typename T, int N, int M>
-__global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src, Cx<T>* C, int nkeep, int pitch) {
+__global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src, const T* sc, Cx<T>* C,
+                                                int nkeep, int pitch) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
     Cx<T>* A = sw + N;
@@ -369,7 +373,13 @@ __global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src
         const int l = q / N, e = q % N;
         const T* row = src + 2 * (pair0 + l) * N;
         const bool ok = pair0 + l < pairs;
-        A[e * (M + 1) + l] = Cx<T>{ok ? row[e] : (T)0, ok ? row[N + e] : (T)0};
+        Cx<T> v = {ok ? row[e] : (T)0, ok ? row[N + e] : (T)0};
+        if (sc && ok) {
+            const T* f = sc + 2 * (pair0 + l) * N;
+            v.re *= f[e];
+            v.im *= f[N + e];
+        }
+        A[e * (M + 1) + l] = v;
     }
     __syncthreads();
     Cx<T>* R = sstage<T, N, M, false, 0>(A, B, sw);
@@ -386,10 +396,11 @@ __global__ void __launch_bounds__(256) ks_x_fwd(Geo g, const T* tw, const T* src
 // x pass, inverse, two real rows per complex line (Z = A + i B with A and B
 // extended by Hermitian symmetry; the imaginary parts of their zeroth and middle
 // coefficients, which no real row has, are dropped). Coefficients from nkeep on
-// are zero. Planes below *zsplit come from C2 (zsplit null: none does).
+// are zero. Planes below *zsplit come from C2 (zsplit null: none does). The result is
+// multiplied by sc (null: not).
 template <typename T, int N, int M>
 __global__ void __launch_bounds__(256) ks_x_inv(Geo g, const T* tw, const Cx<T>* C, const Cx<T>* C2,
-                                                const int* zsplit, int nkeep, int pitch, T* out) {
+                                                const int* zsplit, int nkeep, int pitch, const T* sc, T* out) {
     extern __shared__ unsigned char smem_raw[];
     Cx<T>* sw = reinterpret_cast<Cx<T>*>(smem_raw);
     Cx<T>* A = sw + N;
@@ -415,7 +426,12 @@ __global__ void __launch_bounds__(256) ks_x_inv(Geo g, const T* tw, const Cx<T>*
     for (int q = threadIdx.x; q < M * N; q += blockDim.x) {
         const int l = q / N, e = q % N;
         if (pair0 + l >= pairs) continue;
-        const Cx<T> v = R[e * (M + 1) + l];
+        Cx<T> v = R[e * (M + 1) + l];
+        if (sc) {
+            const T* f = sc + 2 * (pair0 + l) * N;
+            v.re *= f[e];
+            v.im *= f[N + e];
+        }
         T* row = out + 2 * (pair0 + l) * N;
         row[e] = v.re;
         row[N + e] = v.im;
@@ -583,7 +599,8 @@ constexpr size_t smem_static() { return (size_t)N * sizeof(Cx<T>) * (1 + 2 * ((s
 // one pass of axis `axis` (0 x-forward, 1 y-forward, 2 z-solve, 3 y-inverse, 4 x-inverse) with N
 // known at compile time; returns false if N has no static instance
 template <typename T, int N>
-void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>* C, cudaStream_t s, bool attr) {
+void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, const T* sc, T* out, Cx<T>* C, cudaStream_t s,
+                 bool attr) {
     constexpr int M = lines_static<T, N>();
     constexpr size_t sm = smem_static<T, N>();
     if (attr) {
@@ -600,7 +617,7 @@ void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>*
     const int nxh = g.nx / 2 + 1;
     const long rows = (long)g.ny * g.nz;
     switch (pass) {
-        case 0: ks_x_fwd<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, src, C, nxh, nxh); break;
+        case 0: ks_x_fwd<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, src, sc, C, nxh, nxh); break;
         case 1: ks_y<T, N, M, false><<<((nxh + M - 1) / M) * g.nz, 256, sm, s>>>(g, tw, C); break;
         case 2: {
             const T* l0 = sizeof(T) == 8 ? (const T*)p->lam[0] : (const T*)p->lam32[0];
@@ -610,7 +627,7 @@ void static_pass(int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>*
             break;
         }
         case 3: ks_y<T, N, M, true><<<((nxh + M - 1) / M) * g.nz, 256, sm, s>>>(g, tw, C); break;
-        case 4: ks_x_inv<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, C, nullptr, nullptr, nxh, nxh, out); break;
+        case 4: ks_x_inv<T, N, M><<<(int)((rows / 2 + M - 1) / M), 256, sm, s>>>(g, tw, C, nullptr, nullptr, nxh, nxh, sc, out); break;
     }
 }
 
@@ -644,8 +661,8 @@ void band_pass(int pass, FFTPlan* p, const GammaFar* f, bool up, const double* s
         case 0: kb_z_inv<N, M><<<nch * (2 * f->my + 1), 256, sm, s>>>(p->tw64[2], f->mx, f->my, f->mz, up ? su : sa,
                                                                       up ? cu : ca, g.ny); break;
         case 1: kb_y<N, M, true><<<nch * g.nz, 256, sm, s>>>(p->tw64[1], f->mx, f->my, ca, cu, zs); break;
-        case 2: ks_x_inv<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], ca, cu, zs, pitch, pitch, out); break;
-        case 3: ks_x_fwd<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], src, ca, pitch, pitch); break;
+        case 2: ks_x_inv<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], ca, cu, zs, pitch, pitch, nullptr, out); break;
+        case 3: ks_x_fwd<double, N, M><<<nx2, 256, sm, s>>>(g, p->tw64[0], src, nullptr, ca, pitch, pitch); break;
         case 4: kb_y<N, M, false><<<nch * g.nz, 256, sm, s>>>(p->tw64[1], f->mx, f->my, ca, cu, nullptr); break;
         case 5: kb_z_fwd<N, M><<<nch * (2 * f->my + 1), 256, sm, s>>>(p->tw64[2], f->mx, f->my, f->mz, ca,
                                                                       up ? su : sa, g.ny, zs, up ? 1 : 0); break;
@@ -673,28 +690,28 @@ bool dispatch_band(int n, int pass, FFTPlan* p, const GammaFar* f, bool up, cons
 }
 
 template <typename T>
-bool dispatch_pass(int n, int pass, FFTPlan* p, const T* tw, const T* src, T* out, Cx<T>* C, cudaStream_t s,
-                   bool attr) {
+bool dispatch_pass(int n, int pass, FFTPlan* p, const T* tw, const T* src, const T* sc, T* out, Cx<T>* C,
+                   cudaStream_t s, bool attr) {
     switch (n) {
-        case 8: static_pass<T, 8>(pass, p, tw, src, out, C, s, attr); return true;
-        case 12: static_pass<T, 12>(pass, p, tw, src, out, C, s, attr); return true;
-        case 16: static_pass<T, 16>(pass, p, tw, src, out, C, s, attr); return true;
-        case 24: static_pass<T, 24>(pass, p, tw, src, out, C, s, attr); return true;
-        case 32: static_pass<T, 32>(pass, p, tw, src, out, C, s, attr); return true;
-        case 48: static_pass<T, 48>(pass, p, tw, src, out, C, s, attr); return true;
-        case 64: static_pass<T, 64>(pass, p, tw, src, out, C, s, attr); return true;
-        case 96: static_pass<T, 96>(pass, p, tw, src, out, C, s, attr); return true;
-        case 128: static_pass<T, 128>(pass, p, tw, src, out, C, s, attr); return true;
-        case 192: static_pass<T, 192>(pass, p, tw, src, out, C, s, attr); return true;
-        case 256: static_pass<T, 256>(pass, p, tw, src, out, C, s, attr); return true;
-        case 384: static_pass<T, 384>(pass, p, tw, src, out, C, s, attr); return true;
-        case 512: static_pass<T, 512>(pass, p, tw, src, out, C, s, attr); return true;
+        case 8: static_pass<T, 8>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 12: static_pass<T, 12>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 16: static_pass<T, 16>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 24: static_pass<T, 24>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 32: static_pass<T, 32>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 48: static_pass<T, 48>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 64: static_pass<T, 64>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 96: static_pass<T, 96>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 128: static_pass<T, 128>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 192: static_pass<T, 192>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 256: static_pass<T, 256>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 384: static_pass<T, 384>(pass, p, tw, src, sc, out, C, s, attr); return true;
+        case 512: static_pass<T, 512>(pass, p, tw, src, sc, out, C, s, attr); return true;
         default: return false;
     }
 }
 
 template <typename T>
-void run_fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s) {
+void run_fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s, const T* sc) {
     const Geo& g = p->g;
     Cx<T>* C = reinterpret_cast<Cx<T>*>(work);
     const size_t cs = sizeof(Cx<T>);
@@ -710,16 +727,16 @@ void run_fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t 
     const int bz = ((nxh + mz - 1) / mz) * g.ny;
     const size_t sx = smem_bytes(g.nx, mx, cs), sy = smem_bytes(g.ny, my, cs), sz = smem_bytes(g.nz, mz, cs);
     // each pass: the compile-time-size kernel when there is one, else the generic one
-    if (!dispatch_pass<T>(g.nx, 0, p, twx, src, out, C, s, false))
-        k_fft_x_fwd<T><<<bx, 256, sx, s>>>(g, p->ax[0], twx, mx, src, C);
-    if (!dispatch_pass<T>(g.ny, 1, p, twy, src, out, C, s, false))
+    if (!dispatch_pass<T>(g.nx, 0, p, twx, src, sc, out, C, s, false))
+        k_fft_x_fwd<T><<<bx, 256, sx, s>>>(g, p->ax[0], twx, mx, src, sc, C);
+    if (!dispatch_pass<T>(g.ny, 1, p, twy, src, sc, out, C, s, false))
         k_fft_y<T, false><<<by, 256, sy, s>>>(g, p->ax[1], twy, my, C);
-    if (!dispatch_pass<T>(g.nz, 2, p, twz, src, out, C, s, false))
+    if (!dispatch_pass<T>(g.nz, 2, p, twz, src, sc, out, C, s, false))
         k_fft_z_solve<T><<<bz, 256, sz, s>>>(g, p->ax[2], twz, mz, p->lam[0], p->lam[1], p->lam[2], C);
-    if (!dispatch_pass<T>(g.ny, 3, p, twy, src, out, C, s, false))
+    if (!dispatch_pass<T>(g.ny, 3, p, twy, src, sc, out, C, s, false))
         k_fft_y<T, true><<<by, 256, sy, s>>>(g, p->ax[1], twy, my, C);
-    if (!dispatch_pass<T>(g.nx, 4, p, twx, src, out, C, s, false))
-        k_fft_x_inv<T><<<bx, 256, sx, s>>>(g, p->ax[0], twx, mx, C, out);
+    if (!dispatch_pass<T>(g.nx, 4, p, twx, src, sc, out, C, s, false))
+        k_fft_x_inv<T><<<bx, 256, sx, s>>>(g, p->ax[0], twx, mx, C, sc, out);
 }
 
 // allow the dynamic shared memory of every pass (done once, before any capture)
@@ -735,7 +752,7 @@ void set_fft_attributes(const Geo& g) {
     cudaFuncSetAttribute(k_fft_z_solve<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sz);
     const int ns[5] = {g.nx, g.ny, g.nz, g.ny, g.nx};
     for (int pass = 0; pass < 5; ++pass)
-        dispatch_pass<T>(ns[pass], pass, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true);
+        dispatch_pass<T>(ns[pass], pass, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true);
 }
 
 }  // namespace
@@ -803,10 +820,10 @@ void fft_band_forward(FFTPlan* p, const GammaFar& f, const double* src, cudaStre
     if (f.up) dispatch_band(g.nz, 5, p, &f, true, nullptr, nullptr, s);
 }
 
-template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s) {
-    run_fft_poisson<T>(p, src, out, work, s);
+template <typename T> void fft_poisson(FFTPlan* p, const T* src, T* out, void* work, cudaStream_t s, const T* sc) {
+    run_fft_poisson<T>(p, src, out, work, s, sc);
 }
-template void fft_poisson<float>(FFTPlan*, const float*, float*, void*, cudaStream_t);
-template void fft_poisson<double>(FFTPlan*, const double*, double*, void*, cudaStream_t);
+template void fft_poisson<float>(FFTPlan*, const float*, float*, void*, cudaStream_t, const float*);
+template void fft_poisson<double>(FFTPlan*, const double*, double*, void*, cudaStream_t, const double*);
 
 }  // namespace gp

@@ -1290,6 +1290,12 @@ __global__ void k_band_eps(Geo g, const T* eps, int first, int band_nz, T* beps)
 
 // f_band = r - A e_vac on the band's interior planes (full-box operator, periodic)
 template <typename T>
+__global__ void k_rsqrt(long n, const T* src, T* dst) {
+    for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x)
+        dst[t] = rsqrt(src[t]);
+}
+
+template <typename T>
 __global__ void k_band_rhs(Geo g, const T* eps, const T* r, const T* ev, int first, int band_nz, T* fb) {
     const long pl = plane_of(g.nx, g.ny);
     const T hx = (T)g.c2x, hy = (T)g.c2y, hz = (T)g.c2z;
@@ -2043,6 +2049,11 @@ template <typename T> void launch_band_eps(const Geo& g, const T* epsT, int firs
     const long n = plane_of(g.nx, g.ny) * (band_nz + 2);
     k_band_eps<T><<<grid_for(n, 256), 256, 0, s>>>(g, epsT, first, band_nz, beps);
 }
+template <typename T> void launch_rsqrt(long n, const T* src, T* dst, cudaStream_t s) {
+    k_rsqrt<T><<<grid_for(n, 256), 256, 0, s>>>(n, src, dst);
+}
+template void launch_rsqrt<float>(long, const float*, float*, cudaStream_t);
+template void launch_rsqrt<double>(long, const double*, double*, cudaStream_t);
 template <typename T> void launch_band_rhs(const Geo& g, const T* epsT, const T* r, const T* ev, int first,
                                            int band_nz, T* fb, cudaStream_t s) {
     const long rows = (long)g.ny * band_nz;
