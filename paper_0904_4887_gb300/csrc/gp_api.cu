@@ -62,6 +62,8 @@ struct Hier {
     T* cx[16] = {};
     T* cy[16] = {};
     T* cz[16] = {};
+    T* dinv[16] = {};
+    LV<T> fine;                                 // level 0 as the sweeps and products see it (FP64: stored faces)
     T* eps0 = nullptr;                          // owned level-0 cell eps (band only)
     T* x = nullptr; T* r = nullptr; T* p = nullptr; T* q = nullptr; T* z = nullptr;   // PCG, level 0
     T* tmp = nullptr;                           // level-0 ping-pong buffer of the fused sweep
@@ -362,12 +364,15 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
             L.nx = lx; L.ny = ly; L.nz = lz; L.zper = zper;
             L.ihx2 = (T)(1.0 / (hx * hx)); L.ihy2 = (T)(1.0 / (hy * hy)); L.ihz2 = (T)(1.0 / (hz * hz));
             L.cell = (l == 0);
-            L.eps = nullptr; L.cx = L.cy = L.cz = nullptr;
-            if (l > 0) {
+            L.eps = nullptr; L.cx = L.cy = L.cz = L.dinv = nullptr;
+            if (l > 0 || sizeof(T) == 8) {
                 H.cx[l] = alloc_level(H, lx, ly, lz);
                 H.cy[l] = alloc_level(H, lx, ly, lz);
                 H.cz[l] = alloc_level(H, lx, ly, lz);
-                L.cx = H.cx[l]; L.cy = H.cy[l]; L.cz = H.cz[l];
+                if (sizeof(T) == 8) H.dinv[l] = alloc_level(H, lx, ly, lz);
+            }
+            if (l > 0) {
+                L.cx = H.cx[l]; L.cy = H.cy[l]; L.cz = H.cz[l]; L.dinv = H.dinv[l];
                 H.u[l] = alloc_level(H, lx, ly, lz);
                 H.f[l] = alloc_level(H, lx, ly, lz);
             }
@@ -392,6 +397,19 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
         H.ready = true;
     }
     H.lv[0].eps = own_eps ? H.eps0 : eps_level0;
+    H.fine = H.lv[0];
+    if (sizeof(T) == 8) {
+        H.fine.cell = 0;
+        H.fine.cx = H.cx[0]; H.fine.cy = H.cy[0]; H.fine.cz = H.cz[0]; H.fine.dinv = H.dinv[0];
+    }
+}
+
+// first level small enough for the persistent single-CTA kernel (never the finest)
+template <typename T>
+int coarse_block_level(const Hier<T>& H) {
+    for (int l = 1; l < H.L; ++l)
+        if ((long)H.lv[l].nx * H.lv[l].ny * H.lv[l].nz <= coarse_block_points<T>()) return l;
+    return H.L - 1;
 }
 
 // coarse-level face coefficients and the dense coarsest inverse, from level 0's eps
@@ -404,6 +422,13 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
         LV<T>& C = H.lv[l];
         ProfScope ps(c, GP_PROF_SETUP, 1);
         launch_coarsen_faces<T>(F, C.nx, C.ny, C.nz, H.cx[l], H.cy[l], H.cz[l], c->s);
+        GP_CHECK_LAUNCH();
+    }
+    // FP64: the finest level's faces, and every level's inverse diagonal
+    if (sizeof(T) == 8) {
+        ProfScope ps(c, GP_PROF_SETUP, 2);
+        launch_cell_faces<T>(H.lv[0], H.cx[0], H.cy[0], H.cz[0], H.dinv[0], c->s);
+        launch_diag_inverse<T>(H.lv, H.dinv, 1, levels - 1, c->s);
         GP_CHECK_LAUNCH();
     }
     // dense inverse of the coarsest operator
@@ -442,7 +467,7 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
 // kernel allows it, and u is cleared first where it does not.
 template <typename T>
 void smooth_fine(gp_ctx* c, Hier<T>& H, T* u, const T* f, int nu, int first, bool from_zero = false) {
-    const LV<T>& V = H.lv[0];
+    const LV<T>& V = H.fine;
     if (nu <= 0) {
         if (from_zero) GP_CUDA(cudaMemsetAsync(lbase(V, u), 0, level_bytes(V), c->s));
         return;
@@ -495,13 +520,9 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
     // coarse ones, and more of them did not lower the V-cycle count
     auto pre_sweeps = [&](int l) { return l == 1 ? c->prm.nu1 : nuc1; };
     auto post_sweeps = [&](int l) { return l == 1 ? c->prm.nu2 : nuc2; };
-    // first level small enough for the persistent single-CTA kernel (never the finest)
-    int lc = L - 1;
-    for (int l = 1; l < L; ++l) {
-        if ((long)H.lv[l].nx * H.lv[l].ny * H.lv[l].nz <= kCoarseBlockPoints) { lc = l; break; }
-    }
+    const int lc = coarse_block_level(H);
     for (int l = 0; l < lc; ++l) {
-        const LV<T>& V = H.lv[l];
+        const LV<T>& V = l == 0 ? H.fine : H.lv[l];
         T* u = l == 0 ? u0 : H.u[l];
         const T* f = l == 0 ? f0 : H.f[l];
         if (l == 0) {
@@ -533,7 +554,7 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
         }
     }
     for (int l = lc - 1; l >= 0; --l) {
-        const LV<T>& V = H.lv[l];
+        const LV<T>& V = l == 0 ? H.fine : H.lv[l];
         T* u = l == 0 ? u0 : H.u[l];
         const T* f = l == 0 ? f0 : H.f[l];
         {
@@ -650,7 +671,7 @@ void pcg(gp_ctx* c, Hier<T>& H, int iters) {
 
 template <typename T>
 void pcg_body(gp_ctx* c, Hier<T>& H, int iters) {
-    const LV<T>& V = H.lv[0];
+    const LV<T>& V = H.fine;
     GP_CUDA(cudaMemsetAsync(lbase(V, H.x), 0, level_bytes(V), c->s));
     vcycle(c, H, H.z, H.r);
     int cur = 0;
@@ -832,7 +853,7 @@ void split_precondition_body(gp_ctx* c, const T* v, T* z) {
     for (int it = 1; it < c->prm.band_vcycles; ++it) {
         {
             ProfScope ps(c, GP_PROF_MG_FINE, 1);
-            launch_residual<T>(B.lv[0], B.x, B.r, B.q, c->s);
+            launch_residual<T>(B.fine, B.x, B.r, B.q, c->s);
         }
         vcycle(c, B, B.z, B.q);
         ProfScope ps(c, GP_PROF_KRYLOV, 1);
@@ -861,7 +882,7 @@ template <typename T>
 int fgmres_inner(gp_ctx* c, const T* rhs, T* x, int m, double rel_tol) {
     Hier<T>& F = full_hier<T>(c);
     ensure_krylov<T>(c, m);
-    const LV<T>& V0 = F.lv[0];
+    const LV<T>& V0 = F.fine;
     std::vector<double> H((size_t)(m + 1) * m, 0.0), cs(m), sn(m), g(m + 1), y(m), hv(kMaxKrylov + 2);
     auto Hij = [&](int i, int j) -> double& { return H[(size_t)i * m + j]; };
     auto Vp = [&](int j) { return reinterpret_cast<T*>(c->kV[j]); };

@@ -43,6 +43,7 @@ struct LV {
     const T* cy;                  //   c?[i] is the face between i and i+1 along ?
     const T* cz;                  //   cz valid for k = -1 .. nz-1
     int cell;
+    const T* dinv;                // 1 / (sum of a point's face coefficients), or null
 };
 
 struct Atoms {
@@ -390,6 +391,11 @@ template <typename T> void launch_restrict(const LV<T>& F, const T* r, const LV<
 template <typename T> void launch_prolong_add(const LV<T>& F, T* u, const LV<T>& C, const T* uc, cudaStream_t s);
 template <typename T> void launch_coarsen_faces(const LV<T>& F, int nxc, int nyc, int nzc,
                                                 T* cx, T* cy, T* cz, cudaStream_t s);
+// face coefficients and inverse diagonal of a cell level (its eps, walls included) as those of a
+// face-coefficient level
+template <typename T> void launch_cell_faces(const LV<T>& F, T* cx, T* cy, T* cz, T* dinv, cudaStream_t s);
+// the inverse diagonals of the face-coefficient levels l0 .. l1 - 1, one launch
+template <typename T> void launch_diag_inverse(const LV<T>* lv, T* const* dinv, int l0, int l1, cudaStream_t s);
 template <typename T> void launch_coarse_matrix(const LV<T>& C, double* M, cudaStream_t s);
 // the inverse of the dense n x n M into M + n*n; pairs: the one-CTA version in
 // float-pair arithmetic (for an FP32 multigrid), else FP64. Returns the launch count.
@@ -409,7 +415,10 @@ template <typename T> void launch_update_p(const LV<T>& L, T* p, const T* z, con
 template <typename T> void launch_copy_level(const LV<T>& L, T* dst, const T* src, cudaStream_t s);
 
 // the bottom of a V-cycle in one CTA (k_mg.cu): levels l0 .. L-1
-constexpr int kCoarseBlockPoints = 4096;    // levels up to this size run in the persistent kernel
+// Levels up to this size run in the persistent kernel. In FP64 that kernel is bound by its one
+// SM's FP64 pipe, so the line lies lower: a half sweep of 2048 points takes 2.5 us there, and a
+// launch across the SMs 3.5 us; of 4096 points 5 us and 3.5 us.
+template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : 4096; }
 template <typename T>
 struct CoarseSet {
     int l0, L, nc, nu1, nu2;

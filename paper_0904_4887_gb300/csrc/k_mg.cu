@@ -133,14 +133,26 @@ __global__ void k_rbgs(LV<T> L, T* u, const T* f, int color, int init) {
     }
 }
 
-// The same half sweep on a face-coefficient level in FP32, one thread per x-pair
-// with 8-byte loads of the pair and of its y and z neighbour pairs (32-bit
-// index arithmetic).
-__device__ __forceinline__ float2 ld_f2(const float* p, long i) { return *reinterpret_cast<const float2*>(p + i); }
+// The same half sweep on a face-coefficient level, one thread per x-pair with vector
+// loads of the pair and of its y and z neighbour pairs (32-bit index arithmetic). FP32
+// forms the diagonal from the six coefficients; FP64 reads its inverse (L.dinv): a
+// point then takes 8 FP64 instructions (6 products, the difference, the scaling)
+// instead of 13 and a division, and the FP64 pipe, at 1/64 of the FP32 rate, is what
+// bounds it. On the finest FP64 level, whose faces are stored for the same reason
+// (45 instructions and a division when formed from eps), a half sweep of 64 x 64 x 128
+// points went from 23 us to 10 us (profiled), and on 96 x 96 x 192 from 77 us to 20 us.
+template <typename T> struct Two;
+template <> struct Two<float> { using V = float2; };
+template <> struct Two<double> { using V = double2; };
+template <typename T> __device__ __forceinline__ typename Two<T>::V ld_2(const T* p, long i) {
+    return *reinterpret_cast<const typename Two<T>::V*>(p + i);
+}
 
-__global__ void __launch_bounds__(256) k_rbgs_pairs(LV<float> L, float* __restrict__ u, const float* __restrict__ f,
-                                                    int color, int init) {
+template <typename T>
+__global__ void __launch_bounds__(256) k_rbgs_pairs(LV<T> L, T* __restrict__ u, const T* __restrict__ f, int color,
+                                                    int init) {
     griddep_wait();
+    using V = typename Two<T>::V;
     const int nx = L.nx, ny = L.ny, nz = L.nz, np = nx >> 1;
     const long pl = (long)nx * ny;
     const int total = np * ny * nz;
@@ -157,19 +169,55 @@ __global__ void __launch_bounds__(256) k_rbgs_pairs(LV<float> L, float* __restri
         const long dzp = (k == nz - 1 && L.zper) ? -(long)(nz - 1) * pl : pl;
         const long cl = p == 0 ? rb + nx - 1 : c2 - 1;     // x - 1 of the even member
         const long cr = p == np - 1 ? rb : c2 + 2;         // x + 1 of the odd member
-        const float2 uo = ld_f2(u, c2);
-        auto pick = [m](float2 v) { return m ? v.y : v.x; };
-        const float uxm = m ? uo.x : u[cl], uxp = m ? u[cr] : uo.y;
-        const float2 cxo = ld_f2(L.cx, c2);
-        const float cxm = m ? cxo.x : L.cx[cl], cxp = m ? cxo.y : cxo.x;
-        const float cym = pick(ld_f2(L.cy, c2 + dym)), cyp = pick(ld_f2(L.cy, c2));
-        const float czm = pick(ld_f2(L.cz, c2 + dzm)), czp = pick(ld_f2(L.cz, c2));
-        const float sum = init ? 0.f
-                               : cxp * uxp + cxm * uxm + cyp * pick(ld_f2(u, c2 + dyp)) +
-                                     cym * pick(ld_f2(u, c2 + dym)) + czp * pick(ld_f2(u, c2 + dzp)) +
-                                     czm * pick(ld_f2(u, c2 + dzm));
-        const float d = cxp + cxm + cyp + cym + czp + czm;
-        u[c2 + m] = __fdividef(sum - pick(ld_f2(f, c2)), d);
+        const V uo = ld_2(u, c2);
+        auto pick = [m](V v) { return m ? v.y : v.x; };
+        const T uxm = m ? uo.x : u[cl], uxp = m ? u[cr] : uo.y;
+        const V cxo = ld_2(L.cx, c2);
+        const T cxm = m ? cxo.x : L.cx[cl], cxp = m ? cxo.y : cxo.x;
+        const T cym = pick(ld_2(L.cy, c2 + dym)), cyp = pick(ld_2(L.cy, c2));
+        const T czm = pick(ld_2(L.cz, c2 + dzm)), czp = pick(ld_2(L.cz, c2));
+        const T sum = init ? (T)0
+                           : cxp * uxp + cxm * uxm + cyp * pick(ld_2(u, c2 + dyp)) + cym * pick(ld_2(u, c2 + dym)) +
+                                 czp * pick(ld_2(u, c2 + dzp)) + czm * pick(ld_2(u, c2 + dzm));
+        const T rest = sum - pick(ld_2(f, c2));
+        if constexpr (sizeof(T) == 4) u[c2 + m] = __fdividef(rest, cxp + cxm + cyp + cym + czp + czm);
+        else u[c2 + m] = rest * pick(ld_2(L.dinv, c2));
+    }
+}
+
+// faces and inverse diagonal of a cell level: the same products as coefs() forms
+template <typename T>
+__global__ void k_cell_faces(LV<T> F, T* cx, T* cy, T* cz, T* dinv) {
+    LV<T> L = F;
+    const long rows = (long)L.ny * L.nz;
+    const long pl = (long)L.nx * L.ny;
+    for (long row = blockIdx.x; row < rows; row += gridDim.x)
+    for (int i = threadIdx.x; i < L.nx; i += blockDim.x) {
+        const int j = (int)(row % L.ny), k = (int)(row / L.ny);
+        const Nb n = neighbours(L.nx, L.ny, L.nz, L.zper, i, j, k);
+        const Co<T> o = coefs(L, n);
+        cx[n.c] = o.xp;
+        cy[n.c] = o.yp;
+        cz[n.c] = o.zp;
+        if (k == 0 && !L.zper) cz[n.c - pl] = o.zm;         // the lower wall's face
+        dinv[n.c] = (T)1 / (o.xp + o.xm + o.yp + o.ym + o.zp + o.zm);
+    }
+}
+
+template <typename T> struct DiagSet { LV<T> lv[16]; T* dinv[16]; int l0, l1; };
+
+// blockIdx.y is the level
+template <typename T>
+__global__ void k_diag_inverse(DiagSet<T> S) {
+    const LV<T>& L = S.lv[S.l0 + blockIdx.y];
+    T* d = S.dinv[S.l0 + blockIdx.y];
+    const int total = L.nx * L.ny * L.nz;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+        int i, j, k;
+        split3(t, L.nx, L.ny, i, j, k);
+        const Nb n = neighbours(L.nx, L.ny, L.nz, L.zper, i, j, k);
+        const Co<T> o = coefs(L, n);
+        d[n.c] = (T)1 / (o.xp + o.xm + o.yp + o.ym + o.zp + o.zm);
     }
 }
 
@@ -200,15 +248,15 @@ __global__ void k_restrict(LV<T> F, const T* r, LV<T> C, T* fc) {
         for (int dz = -1; dz <= 1; ++dz) {
             int kk = kf + dz;
             if (F.zper) kk = (kk + F.nz) % F.nz;
-            const T wz = dz == 0 ? (T)0.5 : (T)0.25;
             for (int dy = -1; dy <= 1; ++dy) {
                 const int jj = (2 * J + dy + F.ny) % F.ny;
-                const T wy = dy == 0 ? (T)0.5 : (T)0.25;
                 const long base = kk * pl + (long)jj * F.nx;
                 const int ic = 2 * I;
                 const int im = ic == 0 ? F.nx - 1 : ic - 1;
                 const int ip = ic == F.nx - 1 ? 0 : ic + 1;
-                acc += wz * wy * ((T)0.25 * r[base + im] + (T)0.5 * r[base + ic] + (T)0.25 * r[base + ip]);
+                // the weights are powers of two: one product per row carries them all
+                const T w = (T)(0.25 * (dz == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25));
+                acc += w * ((r[base + im] + r[base + ip]) + (T)2 * r[base + ic]);
             }
         }
         fc[I + (long)C.nx * (J + (long)C.ny * K)] = acc;
@@ -263,26 +311,25 @@ __global__ void k_prolong_add(LV<T> F, T* u, LV<T> C, const T* uc) {
     for (int i = threadIdx.x; i < F.nx; i += blockDim.x) {
         const int j = (int)(row % F.ny), k = (int)(row / F.ny);
         int xi[2], yi[2], zi[2];
-        T xw[2], yw[2], zw[2];
-        int nxp, nyp, nzp;
-        if (i & 1) { xi[0] = i >> 1; xi[1] = (xi[0] + 1) % C.nx; xw[0] = xw[1] = (T)0.5; nxp = 2; }
-        else { xi[0] = i >> 1; xw[0] = 1; nxp = 1; }
-        if (j & 1) { yi[0] = j >> 1; yi[1] = (yi[0] + 1) % C.ny; yw[0] = yw[1] = (T)0.5; nyp = 2; }
-        else { yi[0] = j >> 1; yw[0] = 1; nyp = 1; }
+        int nxp = 1, nyp = 1, nzp = 1;
+        T w = 1;                                 // the weights are powers of two: one product carries them all
+        xi[0] = i >> 1;
+        if (i & 1) { xi[1] = (xi[0] + 1) % C.nx; nxp = 2; w *= (T)0.5; }
+        yi[0] = j >> 1;
+        if (j & 1) { yi[1] = (yi[0] + 1) % C.ny; nyp = 2; w *= (T)0.5; }
         const int kk = k - zoff;                 // -1 .. for Dirichlet
         if (kk & 1) {
             zi[0] = (kk - 1) >> 1;               // floor division: -1 -> -1 (the lower wall)
             zi[1] = zi[0] + 1;
             if (C.zper && zi[1] == C.nz) zi[1] = 0;
-            zw[0] = zw[1] = (T)0.5;
             nzp = 2;
-        } else { zi[0] = kk >> 1; zw[0] = 1; nzp = 1; }
+            w *= (T)0.5;
+        } else zi[0] = kk >> 1;
         T acc = 0;
         for (int c = 0; c < nzp; ++c)
             for (int b = 0; b < nyp; ++b)
-                for (int a = 0; a < nxp; ++a)
-                    acc += zw[c] * yw[b] * xw[a] * uc[xi[a] + (long)C.nx * yi[b] + cpl * zi[c]];
-        u[i + (long)F.nx * (j + (long)F.ny * k)] += acc;
+                for (int a = 0; a < nxp; ++a) acc += uc[xi[a] + (long)C.nx * yi[b] + cpl * zi[c]];
+        u[i + (long)F.nx * (j + (long)F.ny * k)] += w * acc;
     }
 }
 
@@ -451,7 +498,8 @@ __global__ void __launch_bounds__(256) k_coarsen_faces_cell(LV<T> F, int nxc, in
 
 // dense matrix of the coarsest operator (row p = point p), periodic levels
 // regularised by -(max|diag|/n) 1 1^T so that mean-zero data give the
-// mean-zero solution
+// mean-zero solution. One CTA; the n^2 shift is written in memory order (a row per thread
+// took 170 us for 396 points)
 template <typename T>
 __global__ void k_coarse_matrix(LV<T> C, double* M) {
     const int n = C.nx * C.ny * C.nz;
@@ -459,7 +507,17 @@ __global__ void k_coarse_matrix(LV<T> C, double* M) {
     if (threadIdx.x == 0) dmax = 0.0;
     __syncthreads();
     for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        for (int q = 0; q < n; ++q) M[(long)p * n + q] = 0.0;
+        int i, j, k;
+        split3(p, C.nx, C.ny, i, j, k);
+        const Co<T> o = coefs(C, neighbours(C.nx, C.ny, C.nz, C.zper, i, j, k));
+        const double d = (double)o.xm + (double)o.xp + (double)o.ym + (double)o.yp + (double)o.zm + (double)o.zp;
+        atomicMax((unsigned long long*)&dmax, __double_as_longlong(d));   // d > 0
+    }
+    __syncthreads();
+    const double s = C.zper ? dmax / n : 0.0;
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) M[e] = -s;
+    __syncthreads();
+    for (int p = threadIdx.x; p < n; p += blockDim.x) {
         int i, j, k;
         split3(p, C.nx, C.ny, i, j, k);
         const Nb nb = neighbours(C.nx, C.ny, C.nz, C.zper, i, j, k);
@@ -468,115 +526,140 @@ __global__ void k_coarse_matrix(LV<T> C, double* M) {
         const double cf[6] = {(double)o.xm, (double)o.xp, (double)o.ym, (double)o.yp, (double)o.zm,
                               (double)o.zp};
         double d = 0.0;
-        for (int s = 0; s < 6; ++s) {
-            d += cf[s];
-            const long q = nbr[s];
-            if (q >= 0 && q < n) M[(long)p * n + q] += cf[s];   // outside: Dirichlet wall (zero)
+        for (int a = 0; a < 6; ++a) {
+            d += cf[a];
+            const long q = nbr[a];
+            if (q >= 0 && q < n) M[(long)p * n + q] += cf[a];   // outside: Dirichlet wall (zero)
         }
         M[(long)p * n + p] -= d;
-        atomicMax((unsigned long long*)&dmax, __double_as_longlong(d));   // d > 0
-    }
-    __syncthreads();
-    if (C.zper) {
-        const double s = dmax / n;
-        for (long e = threadIdx.x; e < (long)n * n; e += blockDim.x) M[e] -= s;
     }
 }
 
 // Inverse by Gauss-Jordan elimination without pivoting. The coarse operator
 // is negative definite (Dirichlet walls, or the periodic operator shifted by
-// -s 1 1^T, whose null space it removes), so every pivot is nonzero and no row
-// exchange is needed. Step `col` subtracts multiples of row col from every
-// other row of [M | W], one CTA per row; row col itself is only read during
-// the step. After the last step M is diagonal and the inverse is W / diag(M).
-__global__ void k_gj_init(double* M, int n, int* status) {
-    double* W = M + (long)n * n;
-    const int r = blockIdx.x;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) W[(long)r * n + q] = (q == r) ? 1.0 : 0.0;
-    if (r == 0 && threadIdx.x == 0) *status = 0;
-}
+// -s 1 1^T, whose null space it removes), so every pivot block is invertible and no
+// row exchange is needed. Above kGjSmemMax points it runs in place over many CTAs, kGjB
+// pivots a step (two launches): with P the inverse of the step's diagonal block,
+//   row block:     M_kj <- P M_kj (j != k), M_kk <- P
+//   other blocks:  M_ij <- M_ij - M_ik M_kj (j != k), M_ik <- -M_ik P,
+// the pivot columns M_ik being copied aside by the first launch, since the second
+// overwrites them. One pivot per launch over [M | I] was n + 2 launches and twice the
+// work: 2.6 ms for 396 points with the operator's assembly, against 1.0 ms.
+constexpr int kGjB = 16;
 
-__global__ void k_gj_step(double* M, int n, int col, int* status) {
-    const int r = blockIdx.x;
-    if (r == col) return;
-    double* W = M + (long)n * n;
-    __shared__ double f;
-    if (threadIdx.x == 0) {
-        const double piv = M[(long)col * n + col];
-        if (!(fabs(piv) > 1e-300)) {
-            f = 0.0;
-            *status = 1;
-        } else {
-            f = M[(long)r * n + col] / piv;
+// the inverse of the kGjB x kGjB (or smaller) block at `col`, thread (r, q) an element; every CTA of
+// the row launch makes it for itself. The pivot's row alone divides (an FP64 division of all the
+// warps held the pipe for most of a step); the others take one FMA a pivot.
+__device__ __forceinline__ void gj_pivot(const double* M, int n, int col, int nb, double (*P)[kGjB + 1], int* status) {
+    __shared__ double f[kGjB], prow[kGjB];
+    const int r = threadIdx.x / kGjB, q = threadIdx.x % kGjB;      // kGjB^2 threads
+    const bool in = r < nb && q < nb;
+    double v = in ? M[(long)(col + r) * n + col + q] : 0.0;
+    if (in) P[r][q] = v;
+    for (int p = 0; p < nb; ++p) {
+        __syncthreads();
+        if (r == p && in) {
+            const double piv = P[p][p];
+            const bool ok = fabs(piv) > 1e-300;
+            if (!ok) *status = 1;
+            const double ip = ok ? 1.0 / piv : 0.0;
+            prow[q] = q == p ? ip : v * ip;
+        }
+        if (q == p && in) f[r] = v;
+        __syncthreads();
+        if (in) {
+            if (r == p) v = prow[q];
+            else v = q == p ? -f[r] * prow[p] : fma(-f[r], prow[q], v);
+            P[r][q] = v;
         }
     }
     __syncthreads();
-    const double fr = f;
-    if (fr == 0.0) return;
-    const double* mc = M + (long)col * n;
-    const double* wc = W + (long)col * n;
-    double* mr = M + (long)r * n;
-    double* wr = W + (long)r * n;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-        mr[q] -= fr * mc[q];
-        wr[q] -= fr * wc[q];
-    }
 }
 
-__global__ void k_gj_finish(double* M, int n) {
-    double* W = M + (long)n * n;
-    const int r = blockIdx.x;
-    __shared__ double inv_d;
-    if (threadIdx.x == 0) inv_d = 1.0 / M[(long)r * n + r];
+// row block: CTA b takes columns b kGjB ..; it also copies its rows' part of the pivot columns to W
+__global__ void __launch_bounds__(kGjB * kGjB) k_gj_row(double* M, double* W, int n, int col, int nb, int* status) {
+    __shared__ double P[kGjB][kGjB + 1], T[kGjB][kGjB + 1];
+    const int r = threadIdx.x / kGjB, q = threadIdx.x % kGjB, j0 = blockIdx.x * kGjB, j = j0 + q;
+    gj_pivot(M, n, col, nb, P, status);
+    // rows j0 .. of the pivot columns, and P, for the second launch
+    if (j0 + r < n && q < nb) W[(long)(j0 + r) * kGjB + q] = M[(long)(j0 + r) * n + col + q];
+    if (blockIdx.x == 0) W[(long)n * kGjB + threadIdx.x] = P[r][q];
+    T[r][q] = r < nb && j < n ? M[(long)(col + r) * n + j] : 0.0;
     __syncthreads();
-    for (int q = threadIdx.x; q < n; q += blockDim.x) W[(long)r * n + q] *= inv_d;
+    if (r >= nb || j >= n || (j >= col && j < col + nb)) return;   // the pivot block: the second launch writes it
+    double acc = 0.0;
+    for (int p = 0; p < nb; ++p) acc += P[r][p] * T[p][q];
+    M[(long)(col + r) * n + j] = acc;
 }
 
-// The same elimination for a small coarsest grid in ONE CTA: [M | I] lives in
-// shared memory (n rows of 2n doubles), each column takes two phases (the
-// row factors, then the row updates) separated by the CTA barrier, and the
-// inverse goes to the second half of M's buffer as in the multi-CTA version.
-constexpr int kGjSmemMax = 110;          // 2 n^2 + n doubles within 200 KB of shared memory
+// the other rows' blocks (grid: column blocks x row blocks) and the pivot columns
+__global__ void __launch_bounds__(kGjB * kGjB) k_gj_update(double* M, const double* W, int n, int col, int nb) {
+    __shared__ double A[kGjB][kGjB + 1], T[kGjB][kGjB + 1];
+    const int r = threadIdx.x / kGjB, q = threadIdx.x % kGjB;
+    const int i = blockIdx.y * kGjB + r, j = blockIdx.x * kGjB + q;
+    const bool pivot_cols = blockIdx.x * kGjB == col;              // col is a multiple of kGjB
+    const bool pivot_rows = blockIdx.y * kGjB == col;
+    if (pivot_rows && !pivot_cols) return;
+    A[r][q] = i < n && q < nb ? W[(long)i * kGjB + q] : 0.0;
+    if (pivot_cols) T[r][q] = W[(long)n * kGjB + threadIdx.x];     // P
+    else T[r][q] = r < nb && j < n ? M[(long)(col + r) * n + j] : 0.0;
+    __syncthreads();
+    if (i >= n || j >= n || (pivot_cols && q >= nb)) return;
+    if (pivot_rows) {
+        M[(long)i * n + j] = T[r][q];
+        return;
+    }
+    double acc = pivot_cols ? 0.0 : M[(long)i * n + j];
+    for (int p = 0; p < nb; ++p) acc -= A[r][p] * T[p][q];
+    M[(long)i * n + j] = acc;
+}
+
+__global__ void k_gj_clear(int* status) { *status = 0; }
+
+// The same elimination for a small coarsest grid in ONE CTA, one pivot at a time in
+// place in shared memory: two phases a pivot (the scaled pivot row and the pivot
+// column aside, then every element), separated by the CTA barrier; the inverse goes
+// to the second half of M's buffer as in the multi-CTA version.
+constexpr int kGjSmemMax = 110;          // n^2 + 2 n doubles within 100 KB of shared memory
 
 __global__ void __launch_bounds__(1024) k_gj_smem(double* M, int n, int* status) {
     extern __shared__ double gja[];
-    double* A = gja;                      // [n][2n]
-    double* fac = gja + 2 * n * n;        // [n]
-    const int w = 2 * n, tid = threadIdx.x;
-    for (int e = tid; e < n * w; e += blockDim.x) {
-        const int r = e / w, q = e - r * w;
-        A[e] = q < n ? M[(long)r * n + q] : (q - n == r ? 1.0 : 0.0);
-    }
+    double* A = gja;                      // [n][n]
+    double* fac = gja + n * n;            // [n] the pivot column
+    double* prow = fac + n;               // [n] the scaled pivot row
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    for (int e = tid; e < n * n; e += blockDim.x) A[e] = M[e];
     if (tid == 0) *status = 0;
     __syncthreads();
-    for (int col = 0; col < n; ++col) {
-        const double piv = A[col * w + col];
-        const bool ok = fabs(piv) > 1e-300;
-        if (!ok && tid == 0) *status = 1;
-        for (int r = tid; r < n; r += blockDim.x) fac[r] = (ok && r != col) ? A[r * w + col] / piv : 0.0;
+    for (int p = 0; p < n; ++p) {
+        if (tid < n) {
+            const double piv = A[p * n + p];
+            const bool ok = fabs(piv) > 1e-300;
+            if (!ok) *status = 1;
+            const double ip = ok ? 1.0 / piv : 0.0;
+            prow[tid] = tid == p ? ip : A[p * n + tid] * ip;
+        } else if (tid >= 512 && tid - 512 < n) {
+            fac[tid - 512] = A[(tid - 512) * n + p];
+        }
         __syncthreads();
-        for (int e = tid; e < n * w; e += blockDim.x) {
-            const int r = e / w, q = e - r * w;
+        for (int r = warp; r < n; r += nw) {
             const double f = fac[r];
-            if (f != 0.0) A[e] -= f * A[col * w + q];
+            for (int q = lane; q < n; q += 32)
+                A[r * n + q] = r == p ? prow[q] : (q == p ? -f * prow[q] : fma(-f, prow[q], A[r * n + q]));
         }
         __syncthreads();
     }
     double* W = M + (long)n * n;
-    for (int e = tid; e < n * n; e += blockDim.x) {
-        const int r = e / n, q = e - r * n;
-        W[e] = A[r * w + n + q] / A[r * w + r];
-    }
+    for (int e = tid; e < n * n; e += blockDim.x) W[e] = A[e];
 }
 
-// The same one-CTA elimination with [M | I] held as float pairs (hi, lo) and
-// every step in pair arithmetic on the FP32 pipe (Dekker's products by FMA,
+// The same one-CTA elimination with every number a float pair (hi, lo) and every
+// step in pair arithmetic on the FP32 pipe (Dekker's products by FMA,
 // Knuth's two-sum, a pair quotient from the float quotient and one correction):
 // about 2^-46 relative per operation. It serves the FP32 multigrid, which stores
 // the inverse in FP32; on one SM the FP64 version is bound by the FP64 pipe
 // (1/64 of the FP32 rate). Rows go to warps and columns to lanes, so no index
-// division; step `col` updates only columns col.. of each row (those before it
-// are already eliminated and stay as they are).
+// division. In place it updates n^2 numbers a pivot: 55 us for 54 points, 71 us over [M | I].
 struct gjp { float hi, lo; };
 __device__ __forceinline__ gjp gjp_quick(float s, float e) {   // |s| >= |e|
     const float t = s + e;
@@ -604,46 +687,41 @@ __device__ __forceinline__ gjp gjp_div(gjp a, gjp b) {
 
 __global__ void __launch_bounds__(1024) k_gj_smem_pairs(double* M, int n, int* status) {
     extern __shared__ float2 gjq[];
-    float2* A = gjq;                      // [n][2n]
-    float2* fac = gjq + 2 * n * n;        // [n]
-    const int w = 2 * n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
-    for (int r = warp; r < n; r += nw)
-        for (int q = lane; q < w; q += 32)
-            A[r * w + q] = q < n ? split_to_float2(M[(long)r * n + q]) : make_float2(q - n == r ? 1.f : 0.f, 0.f);
+    float2* A = gjq;                      // [n][n]
+    float2* fac = gjq + n * n;            // [n] the pivot column
+    float2* prow = fac + n;               // [n] the scaled pivot row
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+    for (int e = tid; e < n * n; e += blockDim.x) A[e] = split_to_float2(M[e]);
     if (tid == 0) *status = 0;
     __syncthreads();
-    for (int col = 0; col < n; ++col) {
-        const float2 pv = A[col * w + col];
-        const gjp piv{pv.x, pv.y};
-        const bool ok = fabsf(piv.hi) > 1e-30f;
-        if (!ok && tid == 0) *status = 1;
-        for (int r = tid; r < n; r += blockDim.x) {
-            const float2 a = A[r * w + col];
-            const gjp f = (ok && r != col) ? gjp_div({a.x, a.y}, piv) : gjp{0.f, 0.f};
-            fac[r] = make_float2(f.hi, f.lo);
+    for (int p = 0; p < n; ++p) {
+        if (tid < n) {
+            const float2 pv = A[p * n + p], a = A[p * n + tid];
+            const bool ok = fabsf(pv.x) > 1e-30f;
+            if (!ok) *status = 1;
+            const gjp v = ok ? gjp_div(tid == p ? gjp{1.f, 0.f} : gjp{a.x, a.y}, {pv.x, pv.y}) : gjp{0.f, 0.f};
+            prow[tid] = make_float2(v.hi, v.lo);
+        } else if (tid >= 512 && tid - 512 < n) {
+            fac[tid - 512] = A[(tid - 512) * n + p];
         }
         __syncthreads();
         for (int r = warp; r < n; r += nw) {
             const float2 fr = fac[r];
-            if (fr.x == 0.f) continue;
-            const gjp f{fr.x, fr.y};
-            for (int q = col + lane; q < w; q += 32) {
-                const float2 a = A[r * w + q], m = A[col * w + q];
-                const gjp v = gjp_sub({a.x, a.y}, gjp_mul(f, {m.x, m.y}));
-                A[r * w + q] = make_float2(v.hi, v.lo);
+            for (int q = lane; q < n; q += 32) {
+                const float2 m = prow[q];
+                if (r == p) {
+                    A[r * n + q] = m;
+                    continue;
+                }
+                const float2 a = q == p ? make_float2(0.f, 0.f) : A[r * n + q];
+                const gjp v = gjp_sub({a.x, a.y}, gjp_mul({fr.x, fr.y}, {m.x, m.y}));
+                A[r * n + q] = make_float2(v.hi, v.lo);
             }
         }
         __syncthreads();
     }
     double* W = M + (long)n * n;
-    for (int r = warp; r < n; r += nw) {
-        const float2 d = A[r * w + r];
-        for (int q = lane; q < n; q += 32) {
-            const float2 a = A[r * w + n + q];
-            const gjp v = gjp_div({a.x, a.y}, {d.x, d.y});
-            W[(long)r * n + q] = (double)v.hi + (double)v.lo;
-        }
-    }
+    for (int e = tid; e < n * n; e += blockDim.x) W[e] = (double)A[e].x + (double)A[e].y;
 }
 
 template <typename T>
@@ -652,9 +730,11 @@ __global__ void k_store_inverse(const double* W, long nn, T* inv) {
         inv[e] = (T)W[e];
 }
 
-// u = inv * f on the coarsest level (periodic: f projected to mean zero first)
+// u = inv * f on the coarsest level (periodic: f projected to mean zero first), a warp per row
+// of the inverse and eight rows per CTA; every CTA takes the mean of f for itself (one CTA for
+// all the rows spent 39 us on 396 of them in FP64, on one SM's FP64 pipe)
 template <typename T>
-__global__ void k_coarse_solve(LV<T> C, const T* inv, int n, const T* f, T* u) {
+__global__ void __launch_bounds__(256) k_coarse_solve(LV<T> C, const T* inv, int n, const T* f, T* u) {
     __shared__ T fs[kMaxCoarse];
     __shared__ double red[32];
     double loc = 0.0;
@@ -668,9 +748,8 @@ __global__ void k_coarse_solve(LV<T> C, const T* inv, int n, const T* f, T* u) {
     __syncthreads();
     for (int p = threadIdx.x; p < n; p += blockDim.x) fs[p] -= (T)mean;
     __syncthreads();
-    // one warp per row of the inverse: coalesced loads, a warp reduction
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int p = threadIdx.x >> 5; p < n; p += nw) {
+    for (int p = blockIdx.x * nw + (threadIdx.x >> 5); p < n; p += gridDim.x * nw) {
         const T* row = inv + (long)p * n;
         T acc = 0;
         for (int q = lane; q < n; q += 32) acc += row[q] * fs[q];
@@ -1582,8 +1661,8 @@ __device__ void sm_rbgs(const LV<T>& L, const QDiv& D, T* u, const T* f, int col
         const int zp = c + ((k == nz - 1 && L.zper) ? -(nz - 1) * pl : pl);
         const T cxm = L.cx[xm], cxp = L.cx[c], cym = L.cy[ym], cyp = L.cy[c], czm = L.cz[zm], czp = L.cz[c];
         const T sm = cxp * u[xp] + cxm * u[xm] + cyp * u[yp] + cym * u[ym] + czp * u[zp] + czm * u[zm];
-        const T d = cxp + cxm + cyp + cym + czp + czm;
-        u[c] = (sm - f[c]) / d;
+        if constexpr (sizeof(T) == 8) u[c] = (sm - f[c]) * L.dinv[c];
+        else u[c] = (sm - f[c]) / (cxp + cxm + cyp + cym + czp + czm);
     }
 }
 
@@ -1621,14 +1700,13 @@ __device__ void sm_restrict(const LV<T>& F, const T* r, const LV<T>& C, const QD
         for (int dz = -1; dz <= 1; ++dz) {
             int kk = kf + dz;
             if (F.zper) kk = kk < 0 ? kk + F.nz : (kk >= F.nz ? kk - F.nz : kk);
-            const T wz = dz == 0 ? (T)0.5 : (T)0.25;
 #pragma unroll
             for (int dy = -1; dy <= 1; ++dy) {
                 int jj = 2 * J + dy;
                 jj = jj < 0 ? jj + F.ny : (jj >= F.ny ? jj - F.ny : jj);
-                const T wy = dy == 0 ? (T)0.5 : (T)0.25;
+                const T w = (T)(0.25 * (dz == 0 ? 0.5 : 0.25) * (dy == 0 ? 0.5 : 0.25));   // powers of two
                 const T* row = r + kk * pl + jj * F.nx;
-                acc += wz * wy * ((T)0.25 * row[im] + (T)0.5 * row[ic] + (T)0.25 * row[ip]);
+                acc += w * ((row[im] + row[ip]) + (T)2 * row[ic]);
             }
         }
         fc[t] = acc;
@@ -1643,24 +1721,29 @@ __device__ void sm_prolong_add(const LV<T>& F, const QDiv& DF, T* u, const LV<T>
     for (int t = threadIdx.x; t < np; t += blockDim.x) {
         const int q = qdiv(t, DF.nx), i = t - q * F.nx;
         const int k = qdiv(q, DF.ny), j = q - k * F.ny;
-        const int x0 = i >> 1, x1 = (i & 1) ? (x0 + 1 == C.nx ? 0 : x0 + 1) : x0;
-        const int y0 = j >> 1, y1 = (j & 1) ? (y0 + 1 == C.ny ? 0 : y0 + 1) : y0;
-        const T wx = (i & 1) ? (T)0.5 : (T)1, wy = (j & 1) ? (T)0.5 : (T)1;
+        const bool ox = i & 1, oy = j & 1;
         const int kk = k - zoff;
-        int z0, z1;
-        T wz;
-        if (kk & 1) {
-            z0 = (kk - 1) >> 1;                  // floor division: -1 -> -1 (the lower wall)
-            z1 = z0 + 1;
-            if (C.zper && z1 == C.nz) z1 = 0;
-            wz = (T)0.5;
-        } else { z0 = kk >> 1; z1 = z0; wz = (T)1; }
+        const bool oz = kk & 1;
+        const int x0 = i >> 1, x1 = x0 + 1 == C.nx ? 0 : x0 + 1;
+        const int y0 = j >> 1, y1 = y0 + 1 == C.ny ? 0 : y0 + 1;
+        const int z0 = kk >> 1;                  // floor division: -1 -> -1 (the lower wall)
+        const int z1 = C.zper && z0 + 1 == C.nz ? 0 : z0 + 1;
         auto at = [&](int x, int y, int z) { return uc[x + C.nx * y + cpl * z]; };
-        // with a weight of 1 the second index repeats the first, weighted 0 below
-        const T wx1 = (i & 1) ? wx : (T)0, wy1 = (j & 1) ? wy : (T)0, wz1 = (kk & 1) ? wz : (T)0;
-        const T a0 = wy * (wx * at(x0, y0, z0) + wx1 * at(x1, y0, z0)) + wy1 * (wx * at(x0, y1, z0) + wx1 * at(x1, y1, z0));
-        const T a1 = wy * (wx * at(x0, y0, z1) + wx1 * at(x1, y0, z1)) + wy1 * (wx * at(x0, y1, z1) + wx1 * at(x1, y1, z1));
-        u[t] += wz * a0 + wz1 * a1;
+        auto line = [&](int y, int z) { return ox ? at(x0, y, z) + at(x1, y, z) : at(x0, y, z); };
+        auto plane = [&](int z) { return oy ? line(y0, z) + line(y1, z) : line(y0, z); };
+        if constexpr (sizeof(T) == 8) {
+            // the weights are powers of two: one product carries them all
+            const T w = (ox ? (T)0.5 : (T)1) * (oy ? (T)0.5 : (T)1) * (oz ? (T)0.5 : (T)1);
+            u[t] += w * (oz ? plane(z0) + plane(z1) : plane(z0));
+        } else {
+            // FP32: no branches; with a weight of 1 the second index repeats the first, weighted 0
+            const int xb = ox ? x1 : x0, yb = oy ? y1 : y0, zb = oz ? z1 : z0;
+            const T wx = ox ? (T)0.5 : (T)1, wy = oy ? (T)0.5 : (T)1, wz = oz ? (T)0.5 : (T)1;
+            const T wx1 = ox ? wx : (T)0, wy1 = oy ? wy : (T)0, wz1 = oz ? wz : (T)0;
+            const T a0 = wy * (wx * at(x0, y0, z0) + wx1 * at(xb, y0, z0)) + wy1 * (wx * at(x0, yb, z0) + wx1 * at(xb, yb, z0));
+            const T a1 = wy * (wx * at(x0, y0, zb) + wx1 * at(xb, y0, zb)) + wy1 * (wx * at(x0, yb, zb) + wx1 * at(xb, yb, zb));
+            u[t] += wz * a0 + wz1 * a1;
+        }
     }
 }
 
@@ -1683,6 +1766,8 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
             v.cx = q + pl; q += P;
             v.cy = q + pl; q += P;
             v.cz = q + pl; q += P;
+            v.dinv = nullptr;
+            if (sizeof(T) == 8 && l < S.L - 1) { v.dinv = q; q += pl * G.nz; }
             su[l] = q + pl; q += P;
             sf[l] = q + pl; q += P;
             sr[l] = nullptr;
@@ -1702,6 +1787,10 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
         T* ff = sf[l] - pl;
         T* rr = sr[l] ? sr[l] - pl : nullptr;
         const T* gf = S.f[l] - pl;
+        if (sizeof(T) == 8 && l < S.L - 1) {
+            T* dd = const_cast<T*>(lv[l].dinv);
+            for (long t = threadIdx.x; t < P - 2 * pl; t += blockDim.x) dd[t] = G.dinv[t];
+        }
         for (long t = threadIdx.x; t < P; t += blockDim.x) {
             x[t] = G.cx[t - pl];
             y[t] = G.cy[t - pl];
@@ -1767,20 +1856,20 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
     for (int l = S.l0; l < S.L; ++l) {
         const LV<T>& G = S.lv[l];
         if (G.cell) return ~(size_t)0;                // the shared copy holds face coefficients only
-        b += (size_t)G.nx * G.ny * (G.nz + 2) * sizeof(T) * (l < S.L - 1 ? 6 : 5);
+        b += (size_t)G.nx * G.ny * sizeof(T) * (l < S.L - 1 ? 6 * (G.nz + 2) + (sizeof(T) == 8 ? G.nz : 0) : 5 * (G.nz + 2));
     }
     return b;
 }
 
 }  // namespace
 
-int gauss_jordan_launches(int n) { return n <= kGjSmemMax ? 1 : n + 2; }
+int gauss_jordan_launches(int n) { return n <= kGjSmemMax ? 1 : 2 * ((n + kGjB - 1) / kGjB) + 1; }
 
 void coarse_vcycle_init() {
     cudaFuncSetAttribute(k_gj_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(double) * (2 * kGjSmemMax * kGjSmemMax + kGjSmemMax)));
+                         (int)(sizeof(double) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
     cudaFuncSetAttribute(k_gj_smem_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(float2) * (2 * kGjSmemMax * kGjSmemMax + kGjSmemMax)));
+                         (int)(sizeof(float2) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
     cudaFuncSetAttribute(k_coarse_vcycle_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
     cudaFuncSetAttribute(k_coarse_vcycle_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
 }
@@ -1900,12 +1989,10 @@ void launch_update_phi(const Geo& g, double* phi, const T* e_full, const T* e_ba
 }
 
 template <typename T> void launch_rbgs(const LV<T>& L, T* u, const T* f, int color, cudaStream_t s, bool init) {
-    if constexpr (sizeof(T) == 4) {
-        if (!L.cell) {
-            const long pairs = (long)(L.nx / 2) * L.ny * L.nz;
-            launch_pdl(k_rbgs_pairs, dim3(grid_for(pairs, 256)), dim3(256), 0, s, L, u, f, color, (int)init);
-            return;
-        }
+    if (!L.cell && (sizeof(T) == 4 || L.dinv)) {
+        const long pairs = (long)(L.nx / 2) * L.ny * L.nz;
+        launch_pdl(k_rbgs_pairs<T>, dim3(grid_for(pairs, 256)), dim3(256), 0, s, L, u, f, color, (int)init);
+        return;
     }
     const long rows = (long)L.ny * L.nz;
     launch_pdl(k_rbgs<T>, dim3(row_blocks(rows)), dim3(row_threads(L.nx / 2)), 0, s, L, u, f, color, (int)init);
@@ -1957,20 +2044,40 @@ template <typename T> void launch_coarsen_faces(const LV<T>& F, int nxc, int nyc
     const long n = (long)nxc * nyc * (nzc + 1);
     k_coarsen_faces<T><<<grid_for(n, 256), 256, 0, s>>>(F, nxc, nyc, nzc, cx, cy, cz);
 }
+template <typename T> void launch_cell_faces(const LV<T>& F, T* cx, T* cy, T* cz, T* dinv, cudaStream_t s) {
+    const long rows = (long)F.ny * F.nz;
+    k_cell_faces<T><<<row_blocks(rows), row_threads(F.nx), 0, s>>>(F, cx, cy, cz, dinv);
+}
+template <typename T> void launch_diag_inverse(const LV<T>* lv, T* const* dinv, int l0, int l1, cudaStream_t s) {
+    if (l1 <= l0) return;
+    DiagSet<T> S;
+    S.l0 = l0;
+    S.l1 = l1;
+    for (int l = l0; l < l1; ++l) { S.lv[l] = lv[l]; S.dinv[l] = dinv[l]; }
+    const long n = (long)lv[l0].nx * lv[l0].ny * lv[l0].nz;
+    k_diag_inverse<T><<<dim3(grid_for(n, 256), l1 - l0), 256, 0, s>>>(S);
+}
 template <typename T> void launch_coarse_matrix(const LV<T>& C, double* M, cudaStream_t s) {
     k_coarse_matrix<T><<<1, 512, 0, s>>>(C, M);
 }
 int launch_gauss_jordan(double* M, int n, int* status, cudaStream_t s, bool pairs) {
     if (n <= kGjSmemMax) {
-        if (pairs) k_gj_smem_pairs<<<1, 1024, sizeof(float2) * (2 * (size_t)n * n + n), s>>>(M, n, status);
-        else k_gj_smem<<<1, 1024, sizeof(double) * (2 * (size_t)n * n + n), s>>>(M, n, status);
+        if (pairs) k_gj_smem_pairs<<<1, 1024, sizeof(float2) * ((size_t)n * n + 2 * n), s>>>(M, n, status);
+        else k_gj_smem<<<1, 1024, sizeof(double) * ((size_t)n * n + 2 * n), s>>>(M, n, status);
         return 1;
     }
-    const int th = n >= 256 ? 256 : 128;
-    k_gj_init<<<n, th, 0, s>>>(M, n, status);
-    for (int col = 0; col < n; ++col) k_gj_step<<<n, th, 0, s>>>(M, n, col, status);
-    k_gj_finish<<<n, th, 0, s>>>(M, n);
-    return n + 2;
+    // in place in M; the pivot columns are copied to the buffer's second half, which the result
+    // then takes (every caller reads the inverse there)
+    double* W = M + (size_t)n * n;
+    const int nblk = (n + kGjB - 1) / kGjB;
+    k_gj_clear<<<1, 1, 0, s>>>(status);
+    for (int b = 0; b < nblk; ++b) {
+        const int col = b * kGjB, nb = n - col < kGjB ? n - col : kGjB;
+        k_gj_row<<<nblk, kGjB * kGjB, 0, s>>>(M, W, n, col, nb, status);
+        k_gj_update<<<dim3(nblk, nblk), kGjB * kGjB, 0, s>>>(M, W, n, col, nb);
+    }
+    cudaMemcpyAsync(W, M, sizeof(double) * (size_t)n * n, cudaMemcpyDeviceToDevice, s);
+    return 2 * nblk + 1;
 }
 template <typename T> void launch_store_inverse(const double* W, int n, T* inv, cudaStream_t s) {
     const long nn = (long)n * n;
@@ -1978,7 +2085,7 @@ template <typename T> void launch_store_inverse(const double* W, int n, T* inv, 
 }
 template <typename T> void launch_coarse_solve(const LV<T>& C, const T* inv, int n, const T* f, T* u,
                                                cudaStream_t s) {
-    k_coarse_solve<T><<<1, 512, 0, s>>>(C, inv, n, f, u);
+    k_coarse_solve<T><<<(n + 7) / 8, 256, 0, s>>>(C, inv, n, f, u);
 }
 template <typename T> void launch_applyA_dot(const LV<T>& L, const T* p, T* q, double* partial, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
@@ -2070,6 +2177,8 @@ template <typename T> void launch_band_rhs(const Geo& g, const T* epsT, const T*
     template void launch_prolong_add<T>(const LV<T>&, T*, const LV<T>&, const T*, cudaStream_t);             \
     template void launch_coarsen_faces<T>(const LV<T>&, int, int, int, T*, T*, T*, cudaStream_t);            \
     template void launch_coarse_matrix<T>(const LV<T>&, double*, cudaStream_t);                              \
+    template void launch_cell_faces<T>(const LV<T>&, T*, T*, T*, T*, cudaStream_t);                          \
+    template void launch_diag_inverse<T>(const LV<T>*, T* const*, int, int, cudaStream_t);                   \
     template void launch_store_inverse<T>(const double*, int, T*, cudaStream_t);                             \
     template void launch_coarse_solve<T>(const LV<T>&, const T*, int, const T*, T*, cudaStream_t);           \
     template void launch_applyA_dot<T>(const LV<T>&, const T*, T*, double*, cudaStream_t);                   \
