@@ -388,6 +388,12 @@ template <typename T> int rb_sweep_resolve(const LV<T>& L, int shape);
 constexpr int kSweepShapeCount = 15;    // 4 x-y tiles + 3 row tiles + 8 warp-specialised row tiles
 template <typename T> void launch_residual(const LV<T>& L, const T* u, const T* f, T* r, cudaStream_t s);
 template <typename T> void launch_restrict(const LV<T>& F, const T* r, const LV<T>& C, T* fc, cudaStream_t s);
+// Middle levels in FP32 (face coefficients): one or two sweeps in one launch, u_out another array
+// than u_in. u_in null: from zero; C not null: from u_in + the interpolated correction uc of C.
+void launch_tile_sweeps(const LV<float>& L, const float* u_in, const float* f, float* u_out, const LV<float>* C,
+                        const float* uc, int sweeps, int first, cudaStream_t s);
+void launch_residual_restrict(const LV<float>& F, const float* u, const float* f, const LV<float>& C, float* fc,
+                              cudaStream_t s);
 template <typename T> void launch_prolong_add(const LV<T>& F, T* u, const LV<T>& C, const T* uc, cudaStream_t s);
 template <typename T> void launch_coarsen_faces(const LV<T>& F, int nxc, int nyc, int nzc,
                                                 T* cx, T* cy, T* cz, cudaStream_t s);
@@ -415,10 +421,12 @@ template <typename T> void launch_update_p(const LV<T>& L, T* p, const T* z, con
 template <typename T> void launch_copy_level(const LV<T>& L, T* dst, const T* src, cudaStream_t s);
 
 // the bottom of a V-cycle in one CTA (k_mg.cu): levels l0 .. L-1
-// Levels up to this size run in the persistent kernel. In FP64 that kernel is bound by its one
-// SM's FP64 pipe, so the line lies lower: a half sweep of 2048 points takes 2.5 us there, and a
+// Levels up to this size run in the persistent kernel. Above it FP32 levels take the fused
+// sweeps, a launch per two sweeps: with the line at 1024 points instead of 4096 a step on
+// 24 x 24 x 48 takes 1.34 ms instead of 1.52, on 96 x 64 x 192 2.93 instead of 2.97. In FP64 the
+// kernel is bound by its one SM's FP64 pipe: a half sweep of 2048 points takes 2.5 us there, a
 // launch across the SMs 3.5 us; of 4096 points 5 us and 3.5 us.
-template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : 4096; }
+template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : 1024; }
 template <typename T>
 struct CoarseSet {
     int l0, L, nc, nu1, nu2;

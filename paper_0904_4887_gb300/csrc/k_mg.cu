@@ -300,6 +300,187 @@ __global__ void __launch_bounds__(256) k_restrict4(LV<float> F, const float* __r
     }
 }
 
+// ------------------------------------------------------------ fused sweeps of the middle levels
+// NS red-black sweeps of a face-coefficient level in one launch (FP32). A CTA takes an
+// 8 x 8 x 8 tile with a halo of 2 NS points and runs all 2 NS half sweeps on it, each on a
+// region one point smaller: the halo's updates repeat what the neighbouring CTAs do with
+// the same values, so the result is that of the half sweep per launch. A thread owns an
+// x pair at four planes: its faces, f and inverse diagonals stay in registers, and only u
+// is exchanged, through shared memory (three to four loads an update; with everything in
+// shared memory it was fourteen, and a launch took 6.9 us). On these levels a launch of one
+// half sweep costs 3.5 to 4.3 us whatever its size (launch gap and L2 latency), and the
+// repeated work is cheaper than that.
+// kZero: u starts at zero; kProlong: u starts from u_in plus the interpolated coarse
+// correction. u_out is another array than u_in (neighbours read its halo).
+constexpr int kTile = 8;
+enum TileStart { kPlain = 0, kZero = 1, kProlong = 2 };
+template <int NS> __host__ __device__ constexpr int tile_threads() { return (kTile + 4 * NS) / 2 * (kTile + 4 * NS) * (kTile / 4 + NS); }
+
+template <int NS, int START>
+__global__ void __launch_bounds__(tile_threads<NS>()) k_tile_sweeps(LV<float> L, const float* __restrict__ u_in,
+                                                                    const float* __restrict__ f,
+                                                                    float* __restrict__ u_out, LV<float> C,
+                                                                    const float* __restrict__ uc, int first) {
+    constexpr int H = 2 * NS, W = kTile + 2 * H, P = W * W, NT = tile_threads<NS>(), WC = W / 2 + 1;
+    __shared__ __align__(16) float su[P * W];
+    __shared__ float sc[START == kProlong ? WC * WC * WC : 1];
+    const int nx = L.nx, ny = L.ny, nz = L.nz, tid = threadIdx.x;
+    const int pl = nx * ny;
+    const int i0 = blockIdx.x * kTile - H, j0 = blockIdx.y * kTile - H, k0 = blockIdx.z * kTile - H;
+    const int x = 2 * (tid % (W / 2)), y = (tid / (W / 2)) % W, zb = 4 * (tid / (W / 2 * W));
+    const int i = ((i0 + x) % nx + nx) % nx;
+    const int j = ((j0 + y) % ny + ny) % ny, jm = j == 0 ? ny - 1 : j - 1;
+    int kk[5];                                           // planes zb - 1 .. zb + 3; -2: outside the level
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        const int k = k0 + zb + q - 1;
+        kk[q] = L.zper ? (k % nz + nz) % nz : (k >= -1 && k < nz ? k : -2);
+    }
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 u[4], ff[4], cx[4], cy[4], cym[4], cz[5], di[4];
+    float cxl[4];
+    griddep_wait();
+    cz[0] = kk[0] >= -1 ? ld_2(L.cz, (long)kk[0] * pl + j * nx + i) : zero;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int k = kk[q + 1];
+        u[q] = ff[q] = cx[q] = cy[q] = cym[q] = zero;
+        cxl[q] = 0.f;
+        cz[q + 1] = k >= -1 ? ld_2(L.cz, (long)k * pl + j * nx + i) : zero;      // plane -1: the lower wall's face
+        if (k >= 0) {
+            const long c = (long)k * pl + j * nx + i;
+            cx[q] = ld_2(L.cx, c);
+            cy[q] = ld_2(L.cy, c);
+            cym[q] = ld_2(L.cy, (long)k * pl + jm * nx + i);
+            ff[q] = ld_2(f, c);
+            if constexpr (32 % (W / 2) != 0) cxl[q] = L.cx[i == 0 ? c + nx - 1 : c - 1];
+            if constexpr (START != kZero) u[q] = ld_2(u_in, c);
+        }
+    }
+    if constexpr (START == kProlong) {
+        // the coarse points under the tile, from the floor of its first point on (the tile starts at
+        // even x and y; a Dirichlet level's z is shifted by one: coarse K sits on fine 2K + 1)
+        const int zoff = L.zper ? 0 : 1, ok = (k0 - zoff) & 1;
+        const int I0 = i0 / 2, J0 = j0 / 2, K0 = (k0 - zoff - ok) / 2;
+        for (int t = tid; t < WC * WC * WC; t += NT) {
+            const int a = t % WC, b = (t / WC) % WC, d = t / (WC * WC);
+            const int I = ((I0 + a) % C.nx + C.nx) % C.nx, J = ((J0 + b) % C.ny + C.ny) % C.ny;
+            int K = K0 + d;
+            if (C.zper) K = (K % C.nz + C.nz) % C.nz;
+            sc[t] = C.zper || (K >= 0 && K < C.nz) ? uc[(long)K * C.nx * C.ny + J * C.nx + I] : 0.f;   // walls: zero
+        }
+        __syncthreads();
+        const int a = x / 2, y0 = y >> 1, y1 = (y + 1) >> 1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (kk[q + 1] < 0) continue;
+            const int Z = zb + q + ok, z0 = Z >> 1, z1 = (Z + 1) >> 1;
+            // a repeated index counts twice: every weight is then 1/4 here, 1/2 more along x
+            auto col = [&](int e) {
+                return 0.25f * ((sc[e + WC * (y0 + WC * z0)] + sc[e + WC * (y1 + WC * z0)]) +
+                                (sc[e + WC * (y0 + WC * z1)] + sc[e + WC * (y1 + WC * z1)]));
+            };
+            const float l = col(a), r = col(a + 1);
+            u[q].x += l;
+            u[q].y += 0.5f * (l + r);
+        }
+    }
+    // x - 1 of the pair's first member; at the tile's edge it is never used
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if constexpr (32 % (W / 2) == 0) cxl[q] = __shfl_up_sync(0xffffffffu, cx[q].y, 1);
+        di[q].x = __fdividef(1.f, cxl[q] + cx[q].x + cy[q].x + cym[q].x + cz[q].x + cz[q + 1].x);
+        di[q].y = __fdividef(1.f, cx[q].x + cx[q].y + cy[q].y + cym[q].y + cz[q].y + cz[q + 1].y);
+        *reinterpret_cast<float2*>(su + x + W * y + P * (zb + q)) = u[q];
+    }
+    __syncthreads();
+    const int par = i0 + j0 + k0 + y;                    // the extents are even (a Dirichlet z does not wrap)
+#pragma unroll
+    for (int h = 0; h < 2 * NS; ++h) {
+        const int color = first ^ (h & 1), lo = h + 1;
+        const bool in_y = y >= lo && y < W - lo;
+        // every update of this half sweep reads the other colour only: no ordering among them
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int z = zb + q, m = (color - (par + z)) & 1, c = x + m + W * y + P * z;
+            const bool on = in_y && z >= lo && z < W - lo && x + m >= lo && x + m < W - lo && kk[q + 1] >= 0;
+            if (!on) continue;
+            auto pick = [m](float2 v) { return m ? v.y : v.x; };
+            const float cxm = m ? cx[q].x : cxl[q], cxp = m ? cx[q].y : cx[q].x;
+            float s = 0.f;
+            if (!(START == kZero && h == 0)) {
+                const float in = m ? u[q].x : u[q].y, out = su[m ? c + 1 : c - 1];   // the pair's other member, and beyond
+                s = (m ? cxm : cxp) * in + (m ? cxp : cxm) * out + pick(cy[q]) * su[c + W] + pick(cym[q]) * su[c - W] +
+                    pick(cz[q + 1]) * (q < 3 ? pick(u[q < 3 ? q + 1 : 3]) : su[c + P]) +
+                    pick(cz[q]) * (q > 0 ? pick(u[q > 0 ? q - 1 : 0]) : su[c - P]);
+            }
+            const float v = (s - pick(ff[q])) * pick(di[q]);
+            if (m) u[q].y = v;
+            else u[q].x = v;
+            su[c] = v;
+        }
+        __syncthreads();
+    }
+    if (x >= H && x < H + kTile && y >= H && y < H + kTile && i0 + x < nx && j0 + y < ny) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int z = zb + q, k = k0 + z;
+            if (z >= H && z < H + kTile && k < nz)
+                *reinterpret_cast<float2*>(u_out + (long)k * pl + (j0 + y) * nx + i0 + x) = u[q];
+        }
+    }
+}
+
+// Residual and full weighting in one launch (FP32, face coefficients): a CTA forms the
+// residual on the 17 x 9 x 9 fine points its 8 x 4 x 4 coarse points weight, in shared
+// memory, so the residual is neither written nor read back and one launch gap goes.
+constexpr int kRrX = 8, kRrY = 4, kRrZ = 4;
+
+__global__ void __launch_bounds__(512) k_residual_restrict(LV<float> F, const float* __restrict__ u,
+                                                           const float* __restrict__ f, LV<float> C,
+                                                           float* __restrict__ fc) {
+    constexpr int WX = 2 * kRrX + 1, WY = 2 * kRrY + 1, WZ = 2 * kRrZ + 1;
+    __shared__ float r[WZ][WY][WX + 1];
+    const int nx = F.nx, ny = F.ny, nz = F.nz, pl = nx * ny, zoff = F.zper ? 0 : 1;
+    const int I0 = blockIdx.x * kRrX, J0 = blockIdx.y * kRrY, K0 = blockIdx.z * kRrZ;
+    griddep_wait();
+    for (int t = threadIdx.x; t < WX * WY * WZ; t += 512) {
+        const int x = t % WX, y = (t / WX) % WY, z = t / (WX * WY);
+        int i = 2 * I0 - 1 + x, j = 2 * J0 - 1 + y, k = 2 * K0 + zoff - 1 + z;
+        if (i < 0) i += nx;
+        if (j < 0) j += ny;
+        if (F.zper && k < 0) k += nz;
+        float v = 0.f;
+        if (i < nx && j < ny && k < nz) {                // beyond: a ragged tile's points, not weighted
+            const long c = (long)k * pl + j * nx + i;
+            const long xm = c + (i == 0 ? nx - 1 : -1), xp = c + (i == nx - 1 ? 1 - nx : 1);
+            const long ym = c + (j == 0 ? (ny - 1) * nx : -nx), yp = c + (j == ny - 1 ? -(ny - 1) * nx : nx);
+            const long zm = c + ((k == 0 && F.zper) ? (long)(nz - 1) * pl : -(long)pl);
+            const long zp = c + ((k == nz - 1 && F.zper) ? -(long)(nz - 1) * pl : (long)pl);
+            const float u0 = u[c];
+            v = f[c] - (F.cx[c] * (u[xp] - u0) - F.cx[xm] * (u0 - u[xm]) + F.cy[c] * (u[yp] - u0) -
+                        F.cy[ym] * (u0 - u[ym]) + F.cz[c] * (u[zp] - u0) - F.cz[zm] * (u0 - u[zm]));
+        }
+        r[z][y][x] = v;
+    }
+    __syncthreads();
+    const int t = threadIdx.x;
+    if (t >= kRrX * kRrY * kRrZ) return;
+    const int x = t % kRrX, y = (t / kRrX) % kRrY, z = t / (kRrX * kRrY);
+    const int I = I0 + x, J = J0 + y, K = K0 + z;
+    if (I >= C.nx || J >= C.ny || K >= C.nz) return;
+    float acc = 0.f;
+#pragma unroll
+    for (int dz = 0; dz < 3; ++dz)
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+            const float w = (dz == 1 ? 0.5f : 0.25f) * (dy == 1 ? 0.5f : 0.25f);
+            const float* q = &r[2 * z + dz][2 * y + dy][2 * x];
+            acc += w * (0.25f * q[0] + 0.5f * q[1] + 0.25f * q[2]);
+        }
+    fc[I + (long)C.nx * (J + (long)C.ny * K)] = acc;
+}
+
 // trilinear interpolation of the coarse correction, added to u
 template <typename T>
 __global__ void k_prolong_add(LV<T> F, T* u, LV<T> C, const T* uc) {
@@ -1865,14 +2046,6 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
 
 int gauss_jordan_launches(int n) { return n <= kGjSmemMax ? 1 : 2 * ((n + kGjB - 1) / kGjB) + 1; }
 
-void coarse_vcycle_init() {
-    cudaFuncSetAttribute(k_gj_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(double) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
-    cudaFuncSetAttribute(k_gj_smem_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(float2) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
-    cudaFuncSetAttribute(k_coarse_vcycle_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
-    cudaFuncSetAttribute(k_coarse_vcycle_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
-}
 
 // A launch with programmatic stream serialization (see griddep_wait): the
 // kernel must call griddep_wait() before its first global memory access.
@@ -2011,6 +2184,39 @@ template <typename T> void launch_residual(const LV<T>& L, const T* u, const T* 
     }
     const long rows = (long)L.ny * L.nz;
     launch_pdl(k_residual<T>, dim3(row_blocks(rows)), dim3(row_threads(L.nx)), 0, s, L, u, f, r);
+}
+// up to two sweeps of a middle level in one launch; start: kPlain, kZero or kProlong (C, uc)
+template <int NS, int START>
+void tile_launch(const LV<float>& L, const float* u_in, const float* f, float* u_out, const LV<float>& C,
+                 const float* uc, int first, cudaStream_t s) {
+    const dim3 grid((L.nx + kTile - 1) / kTile, (L.ny + kTile - 1) / kTile, (L.nz + kTile - 1) / kTile);
+    launch_pdl(k_tile_sweeps<NS, START>, grid, dim3(tile_threads<NS>()), 0, s, L, u_in, f, u_out, C, uc, first);
+}
+void coarse_vcycle_init() {
+    cudaFuncSetAttribute(k_gj_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sizeof(double) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
+    cudaFuncSetAttribute(k_gj_smem_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)(sizeof(float2) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
+    cudaFuncSetAttribute(k_coarse_vcycle_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
+    cudaFuncSetAttribute(k_coarse_vcycle_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
+}
+void launch_tile_sweeps(const LV<float>& L, const float* u_in, const float* f, float* u_out, const LV<float>* C,
+                        const float* uc, int sweeps, int first, cudaStream_t s) {
+    const LV<float>& CC = C ? *C : L;
+    if (sweeps == 2) {
+        if (!u_in) tile_launch<2, kZero>(L, u_in, f, u_out, CC, uc, first, s);
+        else if (C) tile_launch<2, kProlong>(L, u_in, f, u_out, CC, uc, first, s);
+        else tile_launch<2, kPlain>(L, u_in, f, u_out, CC, uc, first, s);
+    } else {
+        if (!u_in) tile_launch<1, kZero>(L, u_in, f, u_out, CC, uc, first, s);
+        else if (C) tile_launch<1, kProlong>(L, u_in, f, u_out, CC, uc, first, s);
+        else tile_launch<1, kPlain>(L, u_in, f, u_out, CC, uc, first, s);
+    }
+}
+void launch_residual_restrict(const LV<float>& F, const float* u, const float* f, const LV<float>& C, float* fc,
+                              cudaStream_t s) {
+    const dim3 grid((C.nx + kRrX - 1) / kRrX, (C.ny + kRrY - 1) / kRrY, (C.nz + kRrZ - 1) / kRrZ);
+    launch_pdl(k_residual_restrict, grid, dim3(512), 0, s, F, u, f, C, fc);
 }
 template <typename T> void launch_restrict(const LV<T>& F, const T* r, const LV<T>& C, T* fc, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
