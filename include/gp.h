@@ -244,9 +244,9 @@ gp_status gp_residual6(gp_ctx* ctx, const double* rho_dev, const double* phi_dev
  * *mu_host (may be NULL) receives mu. Stops when ||r||_2 <= tol ||b||_2,
  * r = b - A6 phi - mu eps, b = -4 pi (rho - mean rho) (gp_get_stats has the
  * history). Method: flexible GMRES(restart) in FP64 on the field system with
- * the border eliminated, right-preconditioned by `inner` steps of the 7-point
- * multigrid-preconditioned CG in the context's precision. Uses the eps of the
- * last gp_set_dielectric. Errors: GP_ERR_INVALID_ARG (null array, tol <= 0),
+ * the border eliminated, right-preconditioned by a V-cycle of the 7-point
+ * multigrid in the context's precision (params.inner is not used). Uses the eps
+ * of the last gp_set_dielectric. Errors: GP_ERR_INVALID_ARG (null array, tol <= 0),
  * GP_ERR_STATE (no dielectric), GP_ERR_NOT_NEUTRAL, GP_ERR_NOT_CONVERGED /
  * GP_ERR_DIVERGED (phi holds the last iterate), GP_ERR_OOM (work fields are
  * allocated on first use), GP_ERR_CUDA. */

@@ -74,6 +74,7 @@ struct Hier {
     bool ready = false;
     GraphSlot pcg_g[kMaxInner + 1];             // pcg(iters) on this hierarchy, one graph per count
     GraphSlot solve_g;                          // fixed-count outer solve (graph_outer)
+    GraphSlot cycle_g;                          // one V-cycle, r into x (sixth-order preconditioner)
     const void* solve_phi = nullptr;            // the user buffers solve_g was captured with
     const void* solve_rho = nullptr;
     std::vector<GraphSlot> prec_g;              // split preconditioner into Krylov vector j (band only)
@@ -94,6 +95,7 @@ template <typename T>
 void free_hier(Hier<T>& H) {
     for (GraphSlot& g : H.pcg_g) clear_slot(g);
     clear_slot(H.solve_g);
+    clear_slot(H.cycle_g);
     for (GraphSlot& g : H.prec_g) clear_slot(g);
     for (void* p : H.allocs) cudaFree(p);
     H = Hier<T>();
@@ -1246,23 +1248,24 @@ gp_status solve_impl(gp_ctx* c, const double* rho, double* phi, double tol) {
 // Eliminating the border, the field solves P A6 phi = P b on zero-mean fields,
 // P v = v - (sum v / sum eps) eps (Q v = v - mean(v) and sum(eps lam) = 0 for the
 // adjoint), and the border value is the removed multiple. Flexible GMRES in
-// FP64 on that projected system, right-preconditioned by the 7-point multigrid
-// (`inner` MG-preconditioned CG steps in the context's working precision): both
-// operators discretise div(eps grad), which is self-adjoint, so A7^-1 serves the
-// forward and the transposed system alike. Device scalars used: 40..42 rho
+// FP64 on that projected system, right-preconditioned by one V-cycle of the 7-point
+// multigrid in the context's working precision: both operators discretise
+// div(eps grad), which is self-adjoint, so A7^-1 serves the forward and the transposed
+// system alike. A7 differs from A6, so a better A7^-1 buys little: with 1, 2, 3, 5 and 7
+// steps of MG-preconditioned CG a solve of 64 x 64 x 128 points took 13, 11, 10, 10 and 10
+// GMRES steps, and 12.1, 12.8, 14.2, 18.8 and 23.9 ms with its adjoint and forces (17, 16,
+// 15, 15, 15 steps on 32 x 128 x 64). Device scalars used: 40..42 rho
 // statistics, 44 sum of the last operator output, 45/46 sums of z and eps z,
 // 47 n, 48..50 eps statistics (48 = sum eps).
 constexpr int kS6Rho = 40, kS6Out = 44, kS6Z = 45, kS6N = 47, kS6Eps = 48;
 
-void ensure_fd6(gp_ctx* c, bool transpose) {
+void ensure_fd6(gp_ctx* c) {
     if (!c->f6_r) c->f6_r = (double*)dalloc(c, sizeof(double) * c->n);
-    if (transpose) {
-        if (!c->f6_d1e) c->f6_d1e = (double*)dalloc(c, sizeof(double) * 3 * c->n);
-        if (c->f6_d1e_version != c->eps_version) {
-            ProfScope ps(c, GP_PROF_SETUP, 1);
-            launch_fd6_d1(c->g, c->eps64, nullptr, c->f6_d1e, c->s);
-            c->f6_d1e_version = c->eps_version;
-        }
+    if (!c->f6_d1e) c->f6_d1e = (double*)dalloc(c, sizeof(double) * 3 * c->n);
+    if (c->f6_d1e_version != c->eps_version) {
+        ProfScope ps(c, GP_PROF_SETUP, 1);
+        launch_fd6_d1(c->g, c->eps64, nullptr, c->f6_d1e, c->s);
+        c->f6_d1e_version = c->eps_version;
     }
     GP_CHECK_LAUNCH();
 }
@@ -1274,7 +1277,7 @@ void fd6_operator(gp_ctx* c, const double* x, const double* rho, double sb, doub
     if (transpose)
         launch_fd6_apply_t(c->g, x, c->eps64, c->f6_d1e, rho, sb, c->scal + kS6Rho, sa, y, c->partial, c->s);
     else
-        launch_fd6_apply(c->g, x, c->eps64, rho, sb, c->scal + kS6Rho, sa, y, c->partial, c->s);
+        launch_fd6_apply(c->g, x, c->eps64, c->f6_d1e, rho, sb, c->scal + kS6Rho, sa, y, c->partial, c->s);
     launch_finalize(c->partial, kReduceBlocks, 1, c->scal + kS6Out, c->s);
     if (transpose) launch_fd6_sub_ratio(c->n, y, nullptr, c->scal + kS6Out, c->scal + kS6N, c->s);
     else launch_fd6_sub_ratio(c->n, y, c->eps64, c->scal + kS6Out, c->scal + kS6Eps, c->s);
@@ -1296,7 +1299,8 @@ void fd6_precondition(gp_ctx* c, const double* v, double* z, bool transpose) {
         ProfScope ps(c, GP_PROF_MISC, 1);
         launch_cast_eps<T>(c->n, v, F.r, c->s);
     }
-    pcg<T>(c, F, c->prm.inner);
+    const long key = ((long)c->prm.nu_coarse << 32) | ((long)c->prm.nu1 << 8) | (long)c->prm.nu2;
+    run_graph(c, F.cycle_g, key, [&] { vcycle(c, F, F.x, F.r); });
     ProfScope ps(c, GP_PROF_MISC, 3);
     launch_fd6_to64<T>(c->n, F.x, c->eps64, z, c->partial, c->s);
     launch_finalize(c->partial, kReduceBlocks, 2, c->scal + kS6Z, c->s);
@@ -1311,7 +1315,7 @@ gp_status solve6_impl(gp_ctx* c, const double* rho, double* x, double tol, bool 
     st.outer_iterations = 0; st.inner_iterations = 0; st.vcycles = 0; st.history_len = 0;
     st.residual = NAN;
     const long n = c->n;
-    ensure_fd6(c, transpose);
+    ensure_fd6(c);
     const int m = std::min(std::max(c->prm.restart, 1), kMaxKrylov - 1);
     ensure_krylov<double>(c, m);
     auto Vp = [&](int j) { return reinterpret_cast<double*>(c->kV[j]); };

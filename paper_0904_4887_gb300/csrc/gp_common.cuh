@@ -350,8 +350,8 @@ void launch_residual64(const Geo& g, const double* phi, const double* rho, const
 void launch_residual6(const Geo& g, const double* phi, const double* rho, const double* eps64, double mu,
                       double* r_out, double* partial, cudaStream_t s);
 // sixth-order solve pieces (k_fd6.cu)
-void launch_fd6_apply(const Geo& g, const double* x, const double* eps, const double* rho, double crho,
-                      const double* rsum, double sa, double* y, double* partial, cudaStream_t s);
+void launch_fd6_apply(const Geo& g, const double* x, const double* eps, const double* d1e, const double* rho,
+                      double crho, const double* rsum, double sa, double* y, double* partial, cudaStream_t s);
 void launch_fd6_apply_t(const Geo& g, const double* x, const double* eps, const double* d1e, const double* rho,
                         double crho, const double* rsum, double sa, double* y, double* partial, cudaStream_t s);
 void launch_fd6_d1(const Geo& g, const double* u, const double* w, double* out3, cudaStream_t s);

@@ -22,15 +22,24 @@ constexpr double kB0 = -49.0 / 18.0, kB1 = 27.0 / 18.0, kB2 = -27.0 / 180.0, kB3
 
 __device__ __forceinline__ double fd6_block_sum(double v, double* red) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int t = threadIdx.x + blockDim.x * threadIdx.y, w = t >> 5, l = t & 31;
     if (l == 0) red[w] = v;
     __syncthreads();
     double s = 0.0;
-    if (threadIdx.x < 32) {
-        s = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0;
+    if (t < 32) {
+        s = t < ((blockDim.x * blockDim.y) >> 5) ? red[t] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
-    return s;   // valid in thread 0
+    return s;   // valid in thread (0, 0)
+}
+
+// Row kernels: a block takes several rows at a time when a row is shorter than its 256
+// threads (threads along x, rows along y); with one row per block, rows of 64 points left
+// six warps of eight idle and too few loads in flight: the transposed operator on
+// 64 x 64 x 128 points took 128 us, now 75 (the forward one 106 us, now 62 with stored D1 eps).
+dim3 fd6_block(int nx) {
+    const int tx = nx >= 256 ? 256 : (nx > 64 ? 128 : (nx > 32 ? 64 : 32));
+    return dim3(tx, kReduceThreads / tx);
 }
 
 __device__ __forceinline__ int wrap_up(int v, int n) { return v >= n ? v - n : v; }
@@ -67,7 +76,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_residual6(Geo g, const doubl
     const double ihx2 = g.ihx * g.ihx, ihy2 = g.ihy * g.ihy, ihz2 = g.ihz * g.ihz;
     const double fpi = 4.0 * kPi;
     double s2 = 0.0;
-    for (long row = blockIdx.x; row < (long)ny * nz; row += gridDim.x) {
+    for (long row = blockIdx.x * (long)blockDim.y + threadIdx.y; row < (long)ny * nz; row += (long)gridDim.x * blockDim.y) {
         const int j = (int)(row % ny), k = (int)(row / ny);
         const long base = (long)k * plane + (long)j * nx;
         long ym[3], yp[3], zm[3], zp[3];   // row starts n = 1..3 below / above in y and z
@@ -102,7 +111,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_residual6(Geo g, const doubl
         }
     }
     const double s = fd6_block_sum(s2, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (threadIdx.x + threadIdx.y == 0) partial[blockIdx.x] = s;
 }
 
 // ---------------------------------------------------------------- the solve, its adjoint, the forces
@@ -119,7 +128,8 @@ __global__ void __launch_bounds__(kReduceThreads) k_residual6(Geo g, const doubl
 #define FD6_ROWS_BEGIN                                                             \
     const int nx = g.nx, ny = g.ny, nz = g.nz;                                     \
     const long plane = (long)nx * ny;                                              \
-    for (long row = blockIdx.x; row < (long)ny * nz; row += gridDim.x) {           \
+    for (long row = blockIdx.x * (long)blockDim.y + threadIdx.y; row < (long)ny * nz; \
+         row += (long)gridDim.x * blockDim.y) {                                    \
         const int j = (int)(row % ny), k = (int)(row / ny);                        \
         const long base = (long)k * plane + (long)j * nx;                          \
         long ym[3], yp[3], zm[3], zp[3];                                           \
@@ -169,26 +179,31 @@ __device__ __forceinline__ double s2_prod(const double* __restrict__ a, const do
     return s;
 }
 
-// y = crho (rho - rsum/n) + sa A6 x   (rho may be null); partial[b] = block sum of y
+// y = crho (rho - rsum/n) + sa A6 x   (rho may be null); partial[b] = block sum of y. d1e holds
+// D1 eps per axis, which a solve applies a dozen times: 53 FP64 instructions a point instead of
+// 68 (the FP64 pipe bounds it)
 __global__ void __launch_bounds__(kReduceThreads) k_fd6_apply(Geo g, const double* __restrict__ x,
                                                               const double* __restrict__ eps,
+                                                              const double* __restrict__ d1e,
                                                               const double* __restrict__ rho, double crho,
                                                               const double* rsum, double sa,
                                                               double* __restrict__ y, double* __restrict__ partial) {
     __shared__ double red[32];
     const double ihx2 = g.ihx * g.ihx, ihy2 = g.ihy * g.ihy, ihz2 = g.ihz * g.ihz;
-    const double rmean = rho ? rsum[0] / ((double)g.nx * g.ny * g.nz) : 0.0;
+    const long npts = (long)g.nx * g.ny * g.nz;
+    const double rmean = rho ? rsum[0] / (double)npts : 0.0;
     double acc = 0.0;
     FD6_ROWS_BEGIN
         const double x0 = __ldg(x + c), e0 = __ldg(eps + c);
-        const double a = ihx2 * axis_term(x, eps, x0, e0, mx, px) + ihy2 * axis_term(x, eps, x0, e0, my, py) +
-                         ihz2 * axis_term(x, eps, x0, e0, mz, pz);
+        const double d1 = g.ihx * __ldg(d1e + c) * s1_of(x, mx, px) + g.ihy * __ldg(d1e + npts + c) * s1_of(x, my, py) +
+                          g.ihz * __ldg(d1e + 2 * npts + c) * s1_of(x, mz, pz);
+        const double a = d1 + e0 * (ihx2 * s2_of(x, x0, mx, px) + ihy2 * s2_of(x, x0, my, py) + ihz2 * s2_of(x, x0, mz, pz));
         const double v = (rho ? crho * (__ldg(rho + c) - rmean) : 0.0) + sa * a;
         y[c] = v;
         acc += v;
     FD6_ROWS_END
     const double s = fd6_block_sum(acc, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (threadIdx.x + threadIdx.y == 0) partial[blockIdx.x] = s;
 }
 
 // y = crho (rho - rsum/n) + sa A6^T x with
@@ -216,7 +231,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_fd6_apply_t(Geo g, const dou
         acc += v;
     FD6_ROWS_END
     const double s = fd6_block_sum(acc, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (threadIdx.x + threadIdx.y == 0) partial[blockIdx.x] = s;
 }
 
 // out + a n = D1_a u, a = 0, 1, 2 (1/h included); when w is given, w D1_a u instead
@@ -252,9 +267,13 @@ __global__ void __launch_bounds__(kReduceThreads) k_fd6_weps(Geo g, const double
 
 // y -= (num[0] / den[0]) * (w ? w : 1)
 __global__ void k_fd6_sub_ratio(long n, double* y, const double* w, const double* num, const double* den) {
-    const double r = num[0] / den[0];
+    // one FP64 division a block, not one a thread
+    __shared__ double rs;
+    if (threadIdx.x == 0) rs = num[0] / den[0];
+    __syncthreads();
+    const double r = rs;
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x)
-        y[t] -= r * (w ? w[t] : 1.0);
+        y[t] -= w ? r * w[t] : r;
 }
 
 // dst = (double) src; partial[2b] = sum dst, partial[2b+1] = sum eps dst
@@ -287,7 +306,7 @@ __global__ void __launch_bounds__(kReduceThreads) k_fd6_wrho(long n, const doubl
         a += v;
     }
     const double s = fd6_block_sum(a, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (threadIdx.x + threadIdx.y == 0) partial[blockIdx.x] = s;
 }
 
 // a single device scalar
@@ -301,20 +320,20 @@ int fd6_grid(long n) {
 
 }  // namespace
 
-void launch_fd6_apply(const Geo& g, const double* x, const double* eps, const double* rho, double crho,
-                      const double* rsum, double sa, double* y, double* partial, cudaStream_t s) {
-    k_fd6_apply<<<kReduceBlocks, kReduceThreads, 0, s>>>(g, x, eps, rho, crho, rsum, sa, y, partial);
+void launch_fd6_apply(const Geo& g, const double* x, const double* eps, const double* d1e, const double* rho,
+                      double crho, const double* rsum, double sa, double* y, double* partial, cudaStream_t s) {
+    k_fd6_apply<<<kReduceBlocks, fd6_block(g.nx), 0, s>>>(g, x, eps, d1e, rho, crho, rsum, sa, y, partial);
 }
 void launch_fd6_apply_t(const Geo& g, const double* x, const double* eps, const double* d1e, const double* rho,
                         double crho, const double* rsum, double sa, double* y, double* partial, cudaStream_t s) {
-    k_fd6_apply_t<<<kReduceBlocks, kReduceThreads, 0, s>>>(g, x, eps, d1e, rho, crho, rsum, sa, y, partial);
+    k_fd6_apply_t<<<kReduceBlocks, fd6_block(g.nx), 0, s>>>(g, x, eps, d1e, rho, crho, rsum, sa, y, partial);
 }
 void launch_fd6_d1(const Geo& g, const double* u, const double* w, double* out3, cudaStream_t s) {
-    k_fd6_d1<<<kReduceBlocks, kReduceThreads, 0, s>>>(g, u, w, out3);
+    k_fd6_d1<<<kReduceBlocks, fd6_block(g.nx), 0, s>>>(g, u, w, out3);
 }
 void launch_fd6_weps(const Geo& g, const double* phi, const double* lam, const double* t3, double mu, double* weps,
                      cudaStream_t s) {
-    k_fd6_weps<<<kReduceBlocks, kReduceThreads, 0, s>>>(g, phi, lam, t3, mu, weps);
+    k_fd6_weps<<<kReduceBlocks, fd6_block(g.nx), 0, s>>>(g, phi, lam, t3, mu, weps);
 }
 void launch_fd6_sub_ratio(long n, double* y, const double* w, const double* num, const double* den,
                           cudaStream_t s) {
@@ -333,7 +352,7 @@ void launch_fd6_set(double* slot, double v, cudaStream_t s) { k_fd6_set<<<1, 1, 
 
 void launch_residual6(const Geo& g, const double* phi, const double* rho, const double* eps64, double mu,
                       double* r_out, double* partial, cudaStream_t s) {
-    k_residual6<<<kReduceBlocks, kReduceThreads, 0, s>>>(g, phi, rho, eps64, mu, r_out, partial);
+    k_residual6<<<kReduceBlocks, fd6_block(g.nx), 0, s>>>(g, phi, rho, eps64, mu, r_out, partial);
 }
 
 }  // namespace gp
