@@ -180,7 +180,7 @@ struct gp_ctx {
     int forces_cap = 0;
     double* gmat = nullptr;        // Gauss-Jordan workspace (2 * 512^2)
     double* sw_coef = nullptr;     // switching-function tables (2 * kSwNI * (kSwDeg+1))
-    float4* sw_pack = nullptr;     // their packed FP32 copies (2 * kSwNI * 4)
+    float4* sw_pack = nullptr;     // their packed FP32 copies (2 * kSwNI * kSwVec)
     double sw_key[4] = {0, 0, 0, 0};   // (eps0, r0, w, rcut) the tables were built for
     bool sw_built = false;
     double* rvdw = nullptr;        // van der Waals radii for the kind-1 dielectric
@@ -1676,7 +1676,7 @@ gp_status gp_create(gp_grid grid, gp_cell cell, void* cuda_stream, gp_ctx** out)
         GP_CUDA(cudaMemsetAsync(c->dstatus, 0, sizeof(int) * 4, c->s));
         c->gmat = (double*)dalloc(c, sizeof(double) * 2 * kMaxCoarse * kMaxCoarse);
         c->sw_coef = (double*)dalloc(c, sizeof(double) * 2 * kSwNI * (kSwDeg + 1));
-        c->sw_pack = (float4*)dalloc(c, sizeof(float4) * 2 * kSwNI * 4);
+        c->sw_pack = (float4*)dalloc(c, sizeof(float4) * 2 * kSwNI * kSwVec);
         rb_sweep_init();
         coarse_vcycle_init();
         {
@@ -1822,7 +1822,7 @@ gp_status gp_set_dielectric(gp_ctx* c, const double* atoms_dev, int n_atoms, con
             tb.s = c->sw_coef;
             tb.h = c->sw_coef + (size_t)kSwNI * (kSwDeg + 1);
             tb.s32 = c->sw_pack;
-            tb.h32 = c->sw_pack + (size_t)kSwNI * 4;
+            tb.h32 = c->sw_pack + (size_t)kSwNI * kSwVec;
             tb.s_qlo = (p.r0 - 4.0 * p.w) * (p.r0 - 4.0 * p.w);
             tb.s_qhi = (p.r0 + 6.0 * p.w) * (p.r0 + 6.0 * p.w);
             tb.s_inv_dq = kSwNI / (tb.s_qhi - tb.s_qlo);
@@ -1833,12 +1833,13 @@ gp_status gp_set_dielectric(gp_ctx* c, const double* atoms_dev, int n_atoms, con
             tb.h_dq = (tb.h_qhi - tb.h_qlo) / kSwNI;
             tb.s_qlof = (float)tb.s_qlo; tb.s_dqf = (float)tb.s_dq;
             tb.h_qlof = (float)tb.h_qlo; tb.h_dqf = (float)tb.h_dq;
+            tb.s_tail = (int)std::ceil(((p.r0 + 4.0 * p.w) * (p.r0 + 4.0 * p.w) - tb.s_qlo) * tb.s_inv_dq);
             // they depend on the parameters alone: built again only when those change
             const double key[4] = {p.eps0, p.r0, p.w, p.rcut};
             if (!c->sw_built || std::memcmp(key, c->sw_key, sizeof(key)) != 0) {
                 ProfScope ps(c, GP_PROF_EPS, 1);
                 launch_switch_tables(dp, tb, c->sw_coef, c->sw_coef + (size_t)kSwNI * (kSwDeg + 1), c->sw_pack,
-                                     c->sw_pack + (size_t)kSwNI * 4, c->s);
+                                     c->sw_pack + (size_t)kSwNI * kSwVec, c->s);
                 GP_CHECK_LAUNCH();
                 std::memcpy(c->sw_key, key, sizeof(key));
                 c->sw_built = true;

@@ -183,19 +183,21 @@ inline DielParams make_diel(double eps0, double r0, double w, double rcut, int k
 __host__ __device__ inline long plane_of(int nx, int ny) { return (long)nx * ny; }
 
 // switching-function tables (k_fields.cu): s and h = s'/(s d) as polynomials in q = d^2
-constexpr int kSwNI = 256, kSwDeg = 9;
-// Packed FP32 copies, 16 floats per interval: the low-degree coefficients
-// (below kSwSplitS for s, kSwSplitH for h) as hi/lo pairs, then the rest as
-// single floats (they are small enough that FP32 leaves < 1e-14 relative).
-constexpr int kSwSplitS = 4, kSwSplitH = 6;
+constexpr int kSwNI = 512, kSwDeg = 7;
+// Packed FP32 copies, kSwVec float4 per interval: the kSwSplit lowest coefficients as
+// hi/lo pairs, then the rest as single floats (they are small enough that FP32 leaves
+// < 1e-14 relative). From interval s_tail on (u = (d - r0)/w >= 4) s is within 7.7e-9 of
+// one: there the row holds 1 - s as single floats.
+constexpr int kSwSplit = 4, kSwVec = 3;
 struct SwTables {
     const double* s = nullptr;    // kSwNI x (kSwDeg+1) monomial coefficients, or null (use erfc)
     const double* h = nullptr;
-    const float4* s32 = nullptr;  // kSwNI x 4 packed (see above)
+    const float4* s32 = nullptr;  // kSwNI x kSwVec packed (see above)
     const float4* h32 = nullptr;
     double s_qlo = 0, s_qhi = 0, s_inv_dq = 0, s_dq = 0;
     double h_qlo = 0, h_qhi = 0, h_inv_dq = 0, h_dq = 0;
     float s_qlof = 0, s_dqf = 0, h_qlof = 0, h_dqf = 0;   // FP32 copies, set on the host
+    int s_tail = 0;
 };
 
 // Table coordinates of the separable squared distance, per atom, image digit

@@ -95,47 +95,55 @@ __global__ void k_switch_tables(DielParams p, SwTables tb, double* s_coef, doubl
     const double qlo = is_h ? tb.h_qlo : tb.s_qlo;
     const double dq = is_h ? tb.h_dq : tb.s_dq;
     constexpr int n = kSwDeg + 1;
-    double fv[n], c[n];
-    for (int j = 0; j < n; ++j) {
-        const double xj = cospi((j + 0.5) / n);
-        const double q = qlo + iv * dq + (xj + 1.0) * 0.5 * dq;
-        const double d = sqrt(q);
-        const double u = (d - p.r0) / p.w;
-        const double sv = 0.5 * erfc(-u);
-        fv[j] = is_h ? exp(-u * u) / (p.w * sqrt(kPi)) / (sv * d) : sv;
-    }
-    for (int m = 0; m < n; ++m) {
-        double acc = 0.0;
-        for (int j = 0; j < n; ++j) acc += fv[j] * cospi(m * (j + 0.5) / n);
-        c[m] = acc * 2.0 / n;
-    }
-    c[0] *= 0.5;
-    // monomial coefficients: T_0 = 1, T_1 = t, T_{m+1} = 2 t T_m - T_{m-1}
-    double Tm1[n], Tm[n], mono[n];
-    for (int e = 0; e < n; ++e) { Tm1[e] = 0.0; Tm[e] = 0.0; mono[e] = 0.0; }
-    Tm1[0] = 1.0;                       // T_0
-    Tm[1] = 1.0;                        // T_1
-    mono[0] += c[0];
-    for (int e = 0; e < n; ++e) mono[e] += c[1] * Tm[e];
-    for (int m = 2; m < n; ++m) {
-        double Tn[n];
-        for (int e = 0; e < n; ++e) Tn[e] = (e > 0 ? 2.0 * Tm[e - 1] : 0.0) - Tm1[e];
-        for (int e = 0; e < n; ++e) { mono[e] += c[m] * Tn[e]; Tm1[e] = Tm[e]; Tm[e] = Tn[e]; }
-    }
+    double mono[n];
     double* out = (is_h ? h_coef : s_coef) + (long)iv * n;
+    auto fit = [&](bool tail) {
+        double fv[n], c[n];
+        for (int j = 0; j < n; ++j) {
+            const double xj = cospi((j + 0.5) / n);
+            const double q = qlo + iv * dq + (xj + 1.0) * 0.5 * dq;
+            const double d = sqrt(q);
+            const double u = (d - p.r0) / p.w;
+            const double sv = 0.5 * erfc(tail ? u : -u);
+            fv[j] = is_h ? exp(-u * u) / (p.w * sqrt(kPi)) / (sv * d) : sv;
+        }
+        for (int m = 0; m < n; ++m) {
+            double acc = 0.0;
+            for (int j = 0; j < n; ++j) acc += fv[j] * cospi(m * (j + 0.5) / n);
+            c[m] = acc * 2.0 / n;
+        }
+        c[0] *= 0.5;
+        // monomial coefficients: T_0 = 1, T_1 = t, T_{m+1} = 2 t T_m - T_{m-1}
+        double Tm1[n], Tm[n];
+        for (int e = 0; e < n; ++e) { Tm1[e] = 0.0; Tm[e] = 0.0; mono[e] = 0.0; }
+        Tm1[0] = 1.0;                       // T_0
+        Tm[1] = 1.0;                        // T_1
+        mono[0] += c[0];
+        for (int e = 0; e < n; ++e) mono[e] += c[1] * Tm[e];
+        for (int m = 2; m < n; ++m) {
+            double Tn[n];
+            for (int e = 0; e < n; ++e) Tn[e] = (e > 0 ? 2.0 * Tm[e - 1] : 0.0) - Tm1[e];
+            for (int e = 0; e < n; ++e) { mono[e] += c[m] * Tn[e]; Tm1[e] = Tm[e]; Tm[e] = Tn[e]; }
+        }
+    };
+    fit(false);
     for (int e = 0; e < n; ++e) out[e] = mono[e];
-    float pk[16];
-    const int split = is_h ? kSwSplitH : kSwSplitS;
-    int o = 0;
-    for (int e = 0; e < split; ++e) {
+    const bool tail = !is_h && iv >= tb.s_tail;
+    if (tail) fit(true);                   // 1 - s, single floats
+    const int split = tail ? 0 : kSwSplit;
+    float pk[4 * kSwVec];
+    for (int e = 0; e < n; ++e) {
         const float hi = (float)mono[e];
-        pk[o++] = hi;
-        pk[o++] = (float)(mono[e] - (double)hi);
+        if (e < split) {
+            pk[2 * e] = hi;
+            pk[2 * e + 1] = (float)(mono[e] - (double)hi);
+        } else {
+            pk[split + e] = hi;
+        }
     }
-    for (int e = split; e < n; ++e) pk[o++] = (float)mono[e];
-    while (o < 16) pk[o++] = 0.f;
-    float4* dst = (is_h ? h_pack : s_pack) + 4L * iv;
-    for (int v = 0; v < 4; ++v) dst[v] = make_float4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
+    for (int o = split + n; o < 4 * kSwVec; ++o) pk[o] = 0.f;
+    float4* dst = (is_h ? h_pack : s_pack) + (long)kSwVec * iv;
+    for (int v = 0; v < kSwVec; ++v) dst[v] = make_float4(pk[4 * v], pk[4 * v + 1], pk[4 * v + 2], pk[4 * v + 3]);
 }
 
 __device__ __forceinline__ double sw_eval(const double* __restrict__ coef, double qlo, double inv_dq, double q) {
@@ -405,23 +413,36 @@ __device__ __forceinline__ df df_horner(df acc, df t, float ch, float cl) {
     return df_quick(s, err + e + cl);
 }
 
-// the polynomial of interval k at t from the packed table (SPLIT df coefficients)
-template <int SPLIT>
+// The packed table in shared memory: a warp's pairs fall into up to 32 different rows, and
+// the three 16-byte loads of a row take two to three passes over the banks there against
+// one pass per distinct line through L1.
+constexpr int kSwSmem = kSwNI * kSwVec * (int)sizeof(float4);
+__device__ __forceinline__ void sw_table(float4* dst, const float4* src) {
+    for (int q = threadIdx.x; q < kSwNI * kSwVec; q += blockDim.x) dst[q] = __ldg(src + q);
+}
+
+// the polynomial of interval k at t: kSwSplit df coefficients, then single ones
 __device__ __forceinline__ df sw_poly(const float4* __restrict__ tab, int k, df t) {
-    float c[16];
-    const float4* src = tab + 4 * k;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        const float4 q = __ldg(src + v);
-        c[4 * v] = q.x; c[4 * v + 1] = q.y; c[4 * v + 2] = q.z; c[4 * v + 3] = q.w;
-    }
-    float v = c[2 * SPLIT + (kSwDeg - SPLIT)];
-#pragma unroll
-    for (int e = kSwDeg - 1; e >= SPLIT; --e) v = fmaf(v, t.hi, c[2 * SPLIT + (e - SPLIT)]);
-    df acc = {v, 0.f};
-#pragma unroll
-    for (int e = SPLIT - 1; e >= 0; --e) acc = df_horner(acc, t, c[2 * e], c[2 * e + 1]);
-    return acc;
+    const float4 a = tab[kSwVec * k], b = tab[kSwVec * k + 1], c = tab[kSwVec * k + 2];
+    float v = fmaf(c.w, t.hi, c.z);
+    v = fmaf(v, t.hi, c.y);
+    v = fmaf(v, t.hi, c.x);
+    df acc = df_horner(df{v, 0.f}, t, b.z, b.w);
+    acc = df_horner(acc, t, b.x, b.y);
+    acc = df_horner(acc, t, a.z, a.w);
+    return df_horner(acc, t, a.x, a.y);
+}
+
+// 1 - s of interval k >= s_tail at t, single floats
+__device__ __forceinline__ float sw_poly_tail(const float4* __restrict__ tab, int k, float t) {
+    const float4 a = tab[kSwVec * k], b = tab[kSwVec * k + 1];
+    float v = fmaf(b.w, t, b.z);
+    v = fmaf(v, t, b.y);
+    v = fmaf(v, t, b.x);
+    v = fmaf(v, t, a.w);
+    v = fmaf(v, t, a.z);
+    v = fmaf(v, t, a.y);
+    return fmaf(v, t, a.x);
 }
 
 // ----------------------------------------------------------------- coordinate tables
@@ -463,7 +484,11 @@ __device__ __forceinline__ long ctab_index(const CoordTabs& ct, int a, int im, i
 
 // ----------------------------------------------------------------- eps, tabulated (df64)
 // The same product as k_build_eps, with s from the packed table in df64
-// arithmetic (about 120 FP32 instructions per pair instead of 25 FP64 ones).
+// arithmetic (about 100 FP32 instructions per pair instead of 25 FP64 ones, 40 where
+// s is within 7.7e-9 of one, nearly half of the pairs). Issue-bound (78% of the issue
+// slots); with the table read through L1 (up to 32 lines a load) and all pairs in df
+// the kernel took 0.87 ms on 128 x 128 x 256 points with 144 atoms, now 0.50, and 1.07 ms on
+// 192 x 192 x 384 with 288, now 0.80.
 // Tiles are 32 x 4 x 16 points, each thread taking 4 points along z, so the
 // per-(tile, atom image) staging (table coordinates loaded from the coordinate
 // tables) is shared by 2048 points. The tile first collects its atom images
@@ -488,6 +513,7 @@ __device__ __forceinline__ Tile make_tile_ez(const Geo& g) {
 __global__ void __launch_bounds__(TT) k_build_eps_tab(Geo g, Atoms at, DielParams p, SwTables tb, CoordTabs ct,
                                                       double* eps64, double* pe64, float* eps32,
                                                       double* plane_max) {
+    extern __shared__ __align__(16) float4 swt[];        // the packed table of s
     __shared__ int eai[ECAP][2];                 // (atom, image) of each surviving image
     __shared__ int cn[EB][NS];
     __shared__ df cf[EB][NS];
@@ -522,6 +548,8 @@ __global__ void __launch_bounds__(TT) k_build_eps_tab(Geo g, Atoms at, DielParam
     __syncthreads();
     const int chunk = ne <= ECAP ? max(at.n, 1) : ACHS;
     const int flush_at = ECAP - chunk * 27;
+    if (ne > 0) sw_table(swt, tb.s32);           // read after the barriers below
+    const int tail = tb.s_tail;
     __syncthreads();
     if (threadIdx.x == 0) ne = 0;
     __syncthreads();
@@ -566,6 +594,15 @@ __global__ void __launch_bounds__(TT) k_build_eps_tab(Geo g, Atoms at, DielParam
                             const int cz = TX + TY + tz + 4 * r;
                             const int n = nxy + cn[e][cz];
                             if (n >= kSwNI) continue;               // d >= r0 + 6w: s == 1
+                            if (n >= tail) {
+                                // s = 1 - t, t < 7.7e-9 in FP32 (1e-15 of s): nearly half of the pairs
+                                const float fh = fxy.hi + cf[e][cz].hi;
+                                const int kk = min((int)fh, 2), kq = n + kk;
+                                if (kq >= kSwNI) continue;
+                                const float v = sw_poly_tail(swt, kq, fmaf(2.f, fh - (float)kk, -1.f));
+                                P[r] = df_add(P[r], df{-P[r].hi * v, 0.f});
+                                continue;
+                            }
                             df tl;
                             const int kq = sw_local(n, df_add(fxy, cf[e][cz]), tl);
                             if (kq >= kSwNI) continue;
@@ -576,8 +613,11 @@ __global__ void __launch_bounds__(TT) k_build_eps_tab(Geo g, Atoms at, DielParam
                                 const float d = sqrtf(fmaxf(qq, 0.f));
                                 sv.hi = 0.5f * erfcf((r0f - d) * iwf);
                                 sv.lo = 0.f;
+                            } else if (kq >= tail) {
+                                P[r] = df_add(P[r], df{-P[r].hi * sw_poly_tail(swt, kq, tl.hi), 0.f});
+                                continue;
                             } else {
-                                sv = sw_poly<kSwSplitS>(tb.s32, kq, tl);
+                                sv = sw_poly(swt, kq, tl);
                             }
                             P[r] = df_mul(P[r], sv);
                             if (P[r].hi < tiny) live[r] = false;
@@ -670,12 +710,17 @@ __device__ __forceinline__ df neg_force_weight_df(const Geo& g, const float2* ph
 // loads the table coordinates and displacements of the tile's 32 columns, 4
 // rows and 16 planes from the coordinate tables (FP64-exact, as df), runs over
 // the 2048 points with compensated FP32 sums, and reduces across the warp in
-// df; the CTA then turns every image's sum into FP64 atomics with full warps.
+// df; the CTA then turns every image's sum into FP64 atomics with full warps. What the four
+// points of a column share is formed once, the table is in shared memory, and the tail
+// pairs (two thirds of them, below 5e-6 of the others) are summed in FP32 per image: 1.06 ->
+// 0.68 ms on 128 x 128 x 256 points with 144 atoms, 1.22 -> 0.87 on 192 x 192 x 384 with 288
+// (phi's conversion included).
 constexpr int ECAPF = 384;              // image list capacity of the force kernel
 
 __global__ void __launch_bounds__(TT) k_forces_eps_tab(Geo g, Atoms at, DielParams p, SwTables tb, CoordTabs ct,
                                                        const float2* phid, const double* wext, const double* pe64,
                                                        double* S) {
+    extern __shared__ __align__(16) float4 swt[];        // the packed table of h
     __shared__ df Ws[TX * TY * EZ];              // index tx + TX (ty + TY z)
     __shared__ df eres[ECAPF][3];                // each image's sum, converted to FP64 by a full warp
     __shared__ int eatom[ECAPF];
@@ -700,6 +745,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_tab(Geo g, Atoms at, DielPara
     }
     __syncthreads();
     if (ne == 0) return;
+    sw_table(swt, tb.h32);
     {
         const df c2x = df_from(g.c2x), c2y = df_from(g.c2y), c2z = df_from(g.c2z);
         for (int q = threadIdx.x; q < TX * TY * EZ; q += TT) {
@@ -753,52 +799,64 @@ __global__ void __launch_bounds__(TT) k_forces_eps_tab(Geo g, Atoms at, DielPara
                 }
                 __syncwarp();
                 float sx = 0.f, cx = 0.f, sy = 0.f, cy = 0.f, sz = 0.f, cz = 0.f;
-                for (int blk = 0; blk < 4 * 16; ++blk) {
-                    int tx, ty, tz;
-                    compact_point(blk & 15, lane, tx, ty, tz);
-                    tz += 4 * (blk >> 4);
-                    if (t.i0 + tx >= g.nx || t.j0 + ty >= g.ny || t.k0 + tz >= g.nz) continue;
-                    const int n = wn[warp][tx] + wn[warp][TX + ty] + wn[warp][TX + TY + tz];
-                    df ratio;   // s'(d) / (s(d) d)
-                    if (n >= kSwNI) {
-                        // d >= r0 + 3.5w (the integer parts of the table coordinate alone
-                        // pass its end): culled at rcut on the FP32 distance; inside it
-                        // u >= 3.5 and s = 1 - erfc(u)/2 is 1 to 3.7e-7, so the ratio is
-                        // s'/d in FP32 (the pair is below 5e-6 of one at the switching radius)
-                        const float dx = wd[warp][tx].hi, dy = wd[warp][TX + ty].hi, dz = wd[warp][TX + TY + tz].hi;
-                        const float qq = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        if (!(qq < rc2f)) continue;
-                        const float rs = rsqrtf(qq);          // 1/d
-                        const float uf = (qq * rs - r0f) * iwf;
-                        ratio.hi = spf_norm * exp2f(-1.44269504f * uf * uf) * rs;   // s'/d = spn exp(-u^2)/d
-                        ratio.lo = 0.f;
-                        const df c = df_mul(Ws[tx + TX * (ty + TY * tz)], ratio);
-                        df_acc(sx, cx, c, wd[warp][tx]);
-                        df_acc(sy, cy, c, wd[warp][TX + ty]);
-                        df_acc(sz, cz, c, wd[warp][TX + TY + tz]);
-                        continue;
+                float fx = 0.f, fy = 0.f, fz = 0.f;      // the FP32 tail pairs, below 5e-6 of the others
+                for (int blk = 0; blk < 16; ++blk) {
+                    int tx, ty, tz0;
+                    compact_point(blk, lane, tx, ty, tz0);
+                    if (t.i0 + tx >= g.nx || t.j0 + ty >= g.ny) continue;
+                    // what the column's four points share
+                    const df dx = wd[warp][tx], dy = wd[warp][TX + ty];
+                    const float qxy = fmaf(dx.hi, dx.hi, dy.hi * dy.hi);
+                    if (!(qxy < rc2f)) continue;
+                    const int nxy = wn[warp][tx] + wn[warp][TX + ty];
+                    const df fxy = df_add(wf[warp][tx], wf[warp][TX + ty]);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int tz = tz0 + 4 * r;
+                        if (t.k0 + tz >= g.nz) continue;
+                        const df W = Ws[tx + TX * (ty + TY * tz)];
+                        const df dz = wd[warp][TX + TY + tz];
+                        const int n = nxy + wn[warp][TX + TY + tz];
+                        if (n >= kSwNI) {
+                            // d >= r0 + 3.5w (the integer parts of the table coordinate alone
+                            // pass its end): culled at rcut on the FP32 distance; inside it
+                            // u >= 3.5 and s = 1 - erfc(u)/2 is 1 to 3.7e-7, so the ratio is
+                            // s'/d in FP32 (the pair is below 5e-6 of one at the switching radius)
+                            const float qq = fmaf(dz.hi, dz.hi, qxy);
+                            if (!(qq < rc2f)) continue;
+                            const float rs = rsqrtf(qq);          // 1/d
+                            const float uf = (qq * rs - r0f) * iwf;
+                            const float c = W.hi * spf_norm * exp2f(-1.44269504f * uf * uf) * rs;
+                            fx = fmaf(c, dx.hi, fx);             // s'/d = spn exp(-u^2)/d
+                            fy = fmaf(c, dy.hi, fy);
+                            fz = fmaf(c, dz.hi, fz);
+                            continue;
+                        }
+                        df tl, ratio;   // s'(d) / (s(d) d)
+                        const int kq = sw_local(n, df_add(fxy, wf[warp][TX + TY + tz]), tl);
+                        if (kq >= 0 && kq < kSwNI) {
+                            ratio = sw_poly(swt, kq, tl);
+                        } else {
+                            // |u| > 3.5: the pair is below 5e-6 of one at the switching radius; FP32
+                            const float qq = ((float)kq + 0.5f * (tl.hi + 1.f)) * dq + qlo;
+                            if (!(qq < rc2f && qq > 0.f)) continue;
+                            const float d_ = sqrtf(qq);
+                            const float uf = (d_ - r0f) * iwf;
+                            const float sf = 0.5f * erfcf(-uf);
+                            if (!(sf > 0.f)) continue;           // s underflows: eps - 1 is 0 there, and so is W
+                            const float spf = spf_norm * expf(-uf * uf);
+                            ratio.hi = spf / (sf * d_);
+                            ratio.lo = 0.f;
+                        }
+                        const df c = df_mul(W, ratio);
+                        df_acc(sx, cx, c, dx);
+                        df_acc(sy, cy, c, dy);
+                        df_acc(sz, cz, c, dz);
                     }
-                    const df f = df_add(df_add(wf[warp][tx], wf[warp][TX + ty]), wf[warp][TX + TY + tz]);
-                    df tl;
-                    const int kq = sw_local(n, f, tl);
-                    if (kq >= 0 && kq < kSwNI) {
-                        ratio = sw_poly<kSwSplitH>(tb.h32, kq, tl);
-                    } else {
-                        // |u| > 3.5: the pair is below 5e-6 of one at the switching radius; FP32
-                        const float qq = ((float)kq + 0.5f * (tl.hi + 1.f)) * dq + qlo;
-                        if (!(qq < rc2f && qq > 0.f)) continue;
-                        const float d_ = sqrtf(qq);
-                        const float uf = (d_ - r0f) * iwf;
-                        const float sf = 0.5f * erfcf(-uf);
-                        const float spf = spf_norm * expf(-uf * uf);
-                        ratio.hi = spf / (sf * d_);
-                        ratio.lo = 0.f;
-                    }
-                    const df c = df_mul(Ws[tx + TX * (ty + TY * tz)], ratio);
-                    df_acc(sx, cx, c, wd[warp][tx]);
-                    df_acc(sy, cy, c, wd[warp][TX + ty]);
-                    df_acc(sz, cz, c, wd[warp][TX + TY + tz]);
                 }
+                df_acc(sx, cx, df{fx, 0.f}, df{1.f, 0.f});
+                df_acc(sy, cy, df{fy, 0.f}, df{1.f, 0.f});
+                df_acc(sz, cz, df{fz, 0.f}, df{1.f, 0.f});
                 warp_sum_df(sx, cx); warp_sum_df(sy, cy); warp_sum_df(sz, cz);
                 if (lane == 0) {
                     eres[e][0] = df{sx, cx};
@@ -2156,7 +2214,9 @@ bool launch_build_eps(const Geo& g, Atoms at, DielParams p, const SwTables& tb, 
                       double* pe64, float* eps32, double* plane_max, cudaStream_t s) {
     if (tb.s32) {
         cudaMemsetAsync(plane_max, 0, sizeof(double) * g.nz, s);
-        k_build_eps_tab<<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, tb, ct, eps64, pe64, eps32, plane_max);
+        // the attribute belongs to the device: set on every call rather than remembered per process
+        cudaFuncSetAttribute(k_build_eps_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwSmem);
+        k_build_eps_tab<<<tile_grid_ez(g), TT, kSwSmem, s>>>(g, at, p, tb, ct, eps64, pe64, eps32, plane_max);
         return true;
     }
     k_build_eps<<<tile_grid(g), TT, 0, s>>>(g, at, p, tb, eps64, pe64, eps32);
@@ -2269,8 +2329,10 @@ void launch_energy(const Geo& g, const double* rho, const double* phi, const dou
 void launch_forces_eps(const Geo& g, Atoms at, DielParams p, const SwTables& tb, const CoordTabs& ct,
                        const double* phi, const float2* phid, const double* wext, const double* pe64, double* S,
                        cudaStream_t s) {
-    if (tb.h32) k_forces_eps_tab<<<tile_grid_ez(g), TT, 0, s>>>(g, at, p, tb, ct, phid, wext, pe64, S);
-    else k_forces_eps<<<tile_grid(g), TT, 0, s>>>(g, at, p, tb, phi, wext, pe64, S);
+    if (tb.h32) {
+        cudaFuncSetAttribute(k_forces_eps_tab, cudaFuncAttributeMaxDynamicSharedMemorySize, kSwSmem);
+        k_forces_eps_tab<<<tile_grid_ez(g), TT, kSwSmem, s>>>(g, at, p, tb, ct, phid, wext, pe64, S);
+    } else k_forces_eps<<<tile_grid(g), TT, 0, s>>>(g, at, p, tb, phi, wext, pe64, S);
 }
 
 void launch_forces_rho(const Geo& g, const GaussTabs& gt, const double* phi, float2* phid, double* T,
