@@ -140,7 +140,9 @@ typedef struct {
                                    4, 6, 8 rows; 7 to 14: whole x rows times 6, 4, 6, 4, 16, 14,
                                    14, 12 rows with a producer warp and 2, 2, 4, 3, 2, 4, 2, 2 rows
                                    per thread (shapes 4 to 14 for nx = 64, 96, 128, 192, 256 where
-                                   the tile fits one CTA; otherwise 0) */
+                                   the tile fits one CTA; otherwise 0); -1: two sweeps a launch on
+                                   8x8x8 tiles (FP32 grids of up to 1.2e5 points, unless a
+                                   shape is given) */
     double gamma_cutoff;        /* kinds 1, 2: radius of the Eq. 9 image sum (Angstrom), else 0 */
 } gp_stats;
 

@@ -31,6 +31,7 @@ struct Err {
 
 #define GP_CHECK_LAUNCH() GP_CUDA(cudaGetLastError())
 
+constexpr long kTileFinest = 120000;   // finest levels up to this size take the fused sweeps
 constexpr int kMaxInner = 16;   // PCG iterations one correction may take (adaptive counts included)
 
 // A captured CUDA graph and what replaying it adds to the counters: the
@@ -64,6 +65,7 @@ struct Hier {
     T* cz[16] = {};
     T* dinv[16] = {};
     LV<T> fine;                                 // level 0 as the sweeps and products see it (FP64: stored faces)
+    LV<T> tile0;                                // level 0 with stored faces, for the fused sweeps (small FP32 grids)
     T* eps0 = nullptr;                          // owned level-0 cell eps (band only)
     T* x = nullptr; T* r = nullptr; T* p = nullptr; T* q = nullptr; T* z = nullptr;   // PCG, level 0
     T* tmp = nullptr;                           // level-0 ping-pong buffer of the fused sweep
@@ -367,7 +369,7 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
             L.ihx2 = (T)(1.0 / (hx * hx)); L.ihy2 = (T)(1.0 / (hy * hy)); L.ihz2 = (T)(1.0 / (hz * hz));
             L.cell = (l == 0);
             L.eps = nullptr; L.cx = L.cy = L.cz = L.dinv = nullptr;
-            if (l > 0 || sizeof(T) == 8) {
+            if (l > 0 || sizeof(T) == 8 || (long)lx * ly * lz <= kTileFinest) {
                 H.cx[l] = alloc_level(H, lx, ly, lz);
                 H.cy[l] = alloc_level(H, lx, ly, lz);
                 H.cz[l] = alloc_level(H, lx, ly, lz);
@@ -399,10 +401,11 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
         H.ready = true;
     }
     H.lv[0].eps = own_eps ? H.eps0 : eps_level0;
-    H.fine = H.lv[0];
-    if (sizeof(T) == 8) {
-        H.fine.cell = 0;
-        H.fine.cx = H.cx[0]; H.fine.cy = H.cy[0]; H.fine.cz = H.cz[0]; H.fine.dinv = H.dinv[0];
+    H.fine = H.tile0 = H.lv[0];
+    if (H.cx[0]) {
+        H.tile0.cell = 0;
+        H.tile0.cx = H.cx[0]; H.tile0.cy = H.cy[0]; H.tile0.cz = H.cz[0]; H.tile0.dinv = H.dinv[0];
+        if (sizeof(T) == 8) H.fine = H.tile0;
     }
 }
 
@@ -423,6 +426,18 @@ bool tile_level(const Hier<T>& H, int l) {
     return sizeof(T) == 4 && l > 0 && (long)H.lv[l].nx * H.lv[l].ny * H.lv[l].nz <= 100000;
 }
 
+// Whether the finest level takes them too, from stored faces: FP32 grids of at most kTileFinest
+// points, unless the caller names a smoother tile. A V-cycle then spends three launches on it (sweeps;
+// residual and restriction; interpolation and sweeps) instead of seven. The line by whole-step time
+// (ms, fused / the better x-y tile): 1.23 / 1.29 on 24x24x48, 1.34 / 1.36 on 32x32x64, 1.51 / 1.56 on
+// 48x32x64, 1.68 / 1.71 on 48^3 (110,592 points), but 2.02 / 1.91 on 64x48x64 (196,608) and 2.39 /
+// 2.18 on 64^3, where the x-y tiles fill the chip and read the coefficients once. FP64 (one sweep a
+// launch) loses on every level: 2.05 -> 2.26 ms on 32x32x64, 3.82 -> 4.06 on 64x64x128.
+template <typename T>
+bool tile_finest(const gp_ctx* c, const Hier<T>& H) {
+    return sizeof(T) == 4 && H.cx[0] && c->prm.sweep_shape < 0 && c->prm.nu1 > 0 && c->prm.nu2 > 0;
+}
+
 // coarse-level face coefficients and the dense coarsest inverse, from level 0's eps
 template <typename T>
 void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
@@ -433,6 +448,11 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
         LV<T>& C = H.lv[l];
         ProfScope ps(c, GP_PROF_SETUP, 1);
         launch_coarsen_faces<T>(F, C.nx, C.ny, C.nz, H.cx[l], H.cy[l], H.cz[l], c->s);
+        GP_CHECK_LAUNCH();
+    }
+    if (sizeof(T) == 4 && H.cx[0]) {
+        ProfScope ps(c, GP_PROF_SETUP, 1);
+        launch_cell_faces<T>(H.lv[0], H.cx[0], H.cy[0], H.cz[0], nullptr, c->s);
         GP_CHECK_LAUNCH();
     }
     // FP64: the finest level's faces, and every level's inverse diagonal
@@ -463,6 +483,8 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
     if (sizeof(T) == 4 && c->prm.sweep_shape >= 0) {
         H.sweep_shape = rb_sweep_resolve<T>(H.lv[0], c->prm.sweep_shape);
         c->stats.sweep_shape = H.sweep_shape;
+    } else if (tile_finest(c, H)) {
+        c->stats.sweep_shape = -1;
     } else if (sizeof(T) == 4 && H.sweep_shape < 0) {
         // smoother autotuner: time each tile shape on this level once
         H.sweep_shape = rb_sweep_autotune<T>(H.lv[0], H.x, H.r, H.tmp, c->s);
@@ -534,19 +556,28 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
     const int lc = coarse_block_level(H);
     T* cur[16];                                  // where each level's u is: H.u, or its residual array (fused sweeps)
     for (int l = 0; l < L; ++l) cur[l] = l == 0 ? u0 : H.u[l];
-    auto tiled = [&](int l) { return tile_level(H, l) && pre_sweeps(l) > 0 && post_sweeps(l) > 0; };
+    const bool tile0 = tile_finest(c, H);
+    auto pre_of = [&](int l) { return l == 0 ? c->prm.nu1 : pre_sweeps(l); };
+    auto post_of = [&](int l) { return l == 0 ? c->prm.nu2 : post_sweeps(l); };
+    auto tiled = [&](int l) { return l == 0 ? tile0 : tile_level(H, l) && pre_sweeps(l) > 0 && post_sweeps(l) > 0; };
+    // the fused sweeps go back and forth between two arrays; the finest level's last launch ends in u0
+    auto other = [&](int l, T* p) -> T* {
+        if (l == 0) return p == u0 ? H.tmp : u0;
+        return p == H.u[l] ? H.res[l] : H.u[l];
+    };
+    if (tile0 && ((c->prm.nu1 + 1) / 2 + (c->prm.nu2 + 1) / 2) % 2 == 0) cur[0] = H.tmp;
     for (int l = 0; l < lc; ++l) {
-        const LV<T>& V = l == 0 ? H.fine : H.lv[l];
+        const LV<T>& V = l == 0 ? (tile0 ? H.tile0 : H.fine) : H.lv[l];
         T* u = cur[l];
         const T* f = l == 0 ? f0 : H.f[l];
-        if (l == 0) {
+        if (l == 0 && !tile0) {
             smooth_fine(c, H, u, f, c->prm.nu1, 0, true);
         } else if (tiled(l)) {
             if constexpr (sizeof(T) == 4) {
-                const int nu = pre_sweeps(l);
-                ProfScope ps(c, GP_PROF_MG_COARSE, (nu + 1) / 2 + 1);
+                const int nu = pre_of(l);
+                ProfScope ps(c, l == 0 ? GP_PROF_MG_FINE : GP_PROF_MG_COARSE, (nu + 1) / 2 + 1);
                 for (int it = 0; it < nu; it += 2) {
-                    T* to = it == 0 ? u : (cur[l] == H.u[l] ? H.res[l] : H.u[l]);
+                    T* to = it == 0 ? u : other(l, cur[l]);
                     launch_tile_sweeps(V, it == 0 ? nullptr : cur[l], f, to, nullptr, nullptr, std::min(2, nu - it), 0, c->s);
                     cur[l] = to;
                 }
@@ -587,15 +618,15 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
         }
     }
     for (int l = lc - 1; l >= 0; --l) {
-        const LV<T>& V = l == 0 ? H.fine : H.lv[l];
+        const LV<T>& V = l == 0 ? (tile0 ? H.tile0 : H.fine) : H.lv[l];
         T* u = cur[l];
         const T* f = l == 0 ? f0 : H.f[l];
-        if (l > 0 && tiled(l)) {
+        if (tiled(l)) {
             if constexpr (sizeof(T) == 4) {
-                const int nu = post_sweeps(l);
-                ProfScope ps(c, GP_PROF_MG_COARSE, (nu + 1) / 2);
+                const int nu = post_of(l);
+                ProfScope ps(c, l == 0 ? GP_PROF_MG_FINE : GP_PROF_MG_COARSE, (nu + 1) / 2);
                 for (int it = 0; it < nu; it += 2) {
-                    T* to = cur[l] == H.u[l] ? H.res[l] : H.u[l];
+                    T* to = other(l, cur[l]);
                     launch_tile_sweeps(V, cur[l], f, to, it == 0 ? &H.lv[l + 1] : nullptr, cur[l + 1], std::min(2, nu - it),
                                        1, c->s);
                     cur[l] = to;

@@ -200,7 +200,7 @@ __global__ void k_cell_faces(LV<T> F, T* cx, T* cy, T* cz, T* dinv) {
         cy[n.c] = o.yp;
         cz[n.c] = o.zp;
         if (k == 0 && !L.zper) cz[n.c - pl] = o.zm;         // the lower wall's face
-        dinv[n.c] = (T)1 / (o.xp + o.xm + o.yp + o.ym + o.zp + o.zm);
+        if (dinv) dinv[n.c] = (T)1 / (o.xp + o.xm + o.yp + o.ym + o.zp + o.zm);
     }
 }
 

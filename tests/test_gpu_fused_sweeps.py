@@ -1,4 +1,4 @@
-"""The fused sweeps of the FP32 middle levels (one or two sweeps a launch on tiles
+"""The fused sweeps of the FP32 middle levels and small finest levels (one or two sweeps a launch on tiles
 with a halo, the interpolation in the first launch after the coarse correction,
 residual and restriction in one) against the FP64 hierarchy, which runs every
 half sweep as a launch of its own. The residual after the first outer
