@@ -550,9 +550,11 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
     const int nuc1 = c->prm.nu_coarse > 0 ? c->prm.nu_coarse : c->prm.nu1;   // levels 2 and below
     const int nuc2 = c->prm.nu_coarse > 0 ? c->prm.nu_coarse : c->prm.nu2;
     // level 1 keeps the finest level's counts: its sweeps are the dearest of the
-    // coarse ones, and more of them did not lower the V-cycle count
-    auto pre_sweeps = [&](int l) { return l == 1 ? c->prm.nu1 : nuc1; };
-    auto post_sweeps = [&](int l) { return l == 1 ? c->prm.nu2 : nuc2; };
+    // coarse ones, and more of them did not lower the V-cycle count (a tiny one
+    // takes the coarse counts: there a sweep costs next to nothing)
+    const bool tiny1 = (long)H.lv[1].nx * H.lv[1].ny * H.lv[1].nz <= (sizeof(T) == 8 ? 2048 : 1024);
+    auto pre_sweeps = [&](int l) { return l == 1 && !tiny1 ? c->prm.nu1 : nuc1; };
+    auto post_sweeps = [&](int l) { return l == 1 && !tiny1 ? c->prm.nu2 : nuc2; };
     const int lc = coarse_block_level(H);
     T* cur[16];                                  // where each level's u is: H.u, or its residual array (fused sweeps)
     for (int l = 0; l < L; ++l) cur[l] = l == 0 ? u0 : H.u[l];
@@ -610,9 +612,12 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
         ProfScope ps(c, GP_PROF_MG_COARSE, 1);
         if (lc < L - 1) {
             CoarseSet<T> S;
-            S.l0 = lc; S.L = L; S.nc = H.nc; S.nu1 = nuc1; S.nu2 = nuc2; S.minv = H.minv;
-            for (int l = 0; l < L; ++l) { S.lv[l] = H.lv[l]; S.u[l] = H.u[l]; S.f[l] = H.f[l]; S.r[l] = H.res[l]; }
-            launch_coarse_vcycle<T>(S, c->s);
+            S.l0 = lc; S.L = L; S.nc = H.nc; S.minv = H.minv;
+            for (int l = 0; l < L; ++l) {
+                S.lv[l] = H.lv[l]; S.u[l] = H.u[l]; S.f[l] = H.f[l]; S.r[l] = H.res[l];
+                S.pre[l] = pre_sweeps(l); S.post[l] = post_sweeps(l);
+            }
+            launch_coarse_vcycle(S, c->s);
         } else {
             launch_coarse_solve<T>(H.lv[L - 1], H.minv, H.nc, H.f[L - 1], H.u[L - 1], c->s);
         }

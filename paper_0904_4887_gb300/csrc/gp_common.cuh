@@ -423,22 +423,25 @@ template <typename T> void launch_update_p(const LV<T>& L, T* p, const T* z, con
 template <typename T> void launch_copy_level(const LV<T>& L, T* dst, const T* src, cudaStream_t s);
 
 // the bottom of a V-cycle in one CTA (k_mg.cu): levels l0 .. L-1
-// Levels up to this size run in the persistent kernel. Above it FP32 levels take the fused
-// sweeps, a launch per two sweeps: with the line at 1024 points instead of 4096 a step on
-// 24 x 24 x 48 takes 1.34 ms instead of 1.52, on 96 x 64 x 192 2.93 instead of 2.97. In FP64 the
+// Levels up to this size run in the persistent kernel: in FP32 what a thread's registers hold
+// (with the line at 1024 points instead, and the fused sweeps above it, a step on 24 x 24 x 48 takes
+// 1.25 ms instead of 1.20, on 96 x 64 x 192 2.75 instead of 2.67). In FP64 the
 // kernel is bound by its one SM's FP64 pipe: a half sweep of 2048 points takes 2.5 us there, a
 // launch across the SMs 3.5 us; of 4096 points 5 us and 3.5 us.
-template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : 1024; }
+constexpr int kBottomPoints = 4096;
+template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : kBottomPoints; }
 template <typename T>
 struct CoarseSet {
-    int l0, L, nc, nu1, nu2;
+    int l0, L, nc;
+    int pre[16], post[16];        // sweeps per level
     LV<T> lv[16];
     T* u[16];
     T* f[16];
     T* r[16];
     const T* minv;
 };
-template <typename T> void launch_coarse_vcycle(const CoarseSet<T>& S, cudaStream_t s);
+void launch_coarse_vcycle(const CoarseSet<float>& S, cudaStream_t s);
+void launch_coarse_vcycle(const CoarseSet<double>& S, cudaStream_t s);
 void coarse_vcycle_init();    // allow the shared-memory variant its dynamic shared memory (before any capture)
 
 // dry/wet band (k_mg.cu)

@@ -1674,7 +1674,7 @@ __global__ void k_axpy1(long n, T* x, const T* y) {
 }
 
 // ------------------------------------------------------------ persistent coarse V-cycle
-// The bottom of the V-cycle (levels S.l0 .. S.L-1, each small) in ONE CTA:
+// The FP64 bottom of the V-cycle (levels S.l0 .. S.L-1, each small) in ONE CTA:
 // every smoothing colour, residual, restriction, the coarsest solve and each
 // prolongation is a phase over the level's points, separated by
 // __syncthreads. Replaces a chain of tiny, launch-bound kernels.
@@ -1771,7 +1771,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet<T> S) {
         const int np = V.nx * V.ny * V.nz;
         for (int t = threadIdx.x; t < np; t += blockDim.x) S.u[l][t] = 0;
         __syncthreads();
-        for (int it = 0; it < S.nu1; ++it) {
+        for (int it = 0; it < S.pre[l]; ++it) {
             blk_rbgs(V, S.u[l], S.f[l], 0);
             __syncthreads();
             blk_rbgs(V, S.u[l], S.f[l], 1);
@@ -1807,7 +1807,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet<T> S) {
         const LV<T>& V = S.lv[l];
         blk_prolong_add(V, S.u[l], S.lv[l + 1], S.u[l + 1]);
         __syncthreads();
-        for (int it = 0; it < S.nu2; ++it) {
+        for (int it = 0; it < S.post[l]; ++it) {
             blk_rbgs(V, S.u[l], S.f[l], 1);
             __syncthreads();
             blk_rbgs(V, S.u[l], S.f[l], 0);
@@ -1816,7 +1816,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(CoarseSet<T> S) {
     }
 }
 
-// The same bottom of the V-cycle with the levels' fields and face coefficients
+// The same bottom of the FP64 V-cycle with the levels' fields and face coefficients
 // held in shared memory: each phase then waits on shared-memory latency rather
 // than on an L2 round trip. The arrays keep the padded layout of the global
 // levels (one plane below and one above: the Dirichlet walls of a band); u
@@ -1851,8 +1851,7 @@ __device__ void sm_rbgs(const LV<T>& L, const QDiv& D, T* u, const T* f, int col
         const int zp = c + ((k == nz - 1 && L.zper) ? -(nz - 1) * pl : pl);
         const T cxm = L.cx[xm], cxp = L.cx[c], cym = L.cy[ym], cyp = L.cy[c], czm = L.cz[zm], czp = L.cz[c];
         const T sm = cxp * u[xp] + cxm * u[xm] + cyp * u[yp] + cym * u[ym] + czp * u[zp] + czm * u[zm];
-        if constexpr (sizeof(T) == 8) u[c] = (sm - f[c]) * L.dinv[c];
-        else u[c] = (sm - f[c]) / (cxp + cxm + cyp + cym + czp + czm);
+        u[c] = (sm - f[c]) * L.dinv[c];
     }
 }
 
@@ -1921,19 +1920,9 @@ __device__ void sm_prolong_add(const LV<T>& F, const QDiv& DF, T* u, const LV<T>
         auto at = [&](int x, int y, int z) { return uc[x + C.nx * y + cpl * z]; };
         auto line = [&](int y, int z) { return ox ? at(x0, y, z) + at(x1, y, z) : at(x0, y, z); };
         auto plane = [&](int z) { return oy ? line(y0, z) + line(y1, z) : line(y0, z); };
-        if constexpr (sizeof(T) == 8) {
-            // the weights are powers of two: one product carries them all
-            const T w = (ox ? (T)0.5 : (T)1) * (oy ? (T)0.5 : (T)1) * (oz ? (T)0.5 : (T)1);
-            u[t] += w * (oz ? plane(z0) + plane(z1) : plane(z0));
-        } else {
-            // FP32: no branches; with a weight of 1 the second index repeats the first, weighted 0
-            const int xb = ox ? x1 : x0, yb = oy ? y1 : y0, zb = oz ? z1 : z0;
-            const T wx = ox ? (T)0.5 : (T)1, wy = oy ? (T)0.5 : (T)1, wz = oz ? (T)0.5 : (T)1;
-            const T wx1 = ox ? wx : (T)0, wy1 = oy ? wy : (T)0, wz1 = oz ? wz : (T)0;
-            const T a0 = wy * (wx * at(x0, y0, z0) + wx1 * at(xb, y0, z0)) + wy1 * (wx * at(x0, yb, z0) + wx1 * at(xb, yb, z0));
-            const T a1 = wy * (wx * at(x0, y0, zb) + wx1 * at(xb, y0, zb)) + wy1 * (wx * at(x0, yb, zb) + wx1 * at(xb, yb, zb));
-            u[t] += wz * a0 + wz1 * a1;
-        }
+        // the weights are powers of two: one product carries them all
+        const T w = (ox ? (T)0.5 : (T)1) * (oy ? (T)0.5 : (T)1) * (oz ? (T)0.5 : (T)1);
+        u[t] += w * (oz ? plane(z0) + plane(z1) : plane(z0));
     }
 }
 
@@ -1957,7 +1946,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
             v.cy = q + pl; q += P;
             v.cz = q + pl; q += P;
             v.dinv = nullptr;
-            if (sizeof(T) == 8 && l < S.L - 1) { v.dinv = q; q += pl * G.nz; }
+            if (l < S.L - 1) { v.dinv = q; q += pl * G.nz; }
             su[l] = q + pl; q += P;
             sf[l] = q + pl; q += P;
             sr[l] = nullptr;
@@ -1977,7 +1966,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
         T* ff = sf[l] - pl;
         T* rr = sr[l] ? sr[l] - pl : nullptr;
         const T* gf = S.f[l] - pl;
-        if (sizeof(T) == 8 && l < S.L - 1) {
+        if (l < S.L - 1) {
             T* dd = const_cast<T*>(lv[l].dinv);
             for (long t = threadIdx.x; t < P - 2 * pl; t += blockDim.x) dd[t] = G.dinv[t];
         }
@@ -1992,7 +1981,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
     }
     __syncthreads();
     for (int l = S.l0; l < S.L - 1; ++l) {
-        for (int it = 0; it < S.nu1; ++it) {
+        for (int it = 0; it < S.pre[l]; ++it) {
             sm_rbgs(lv[l], qd[l], su[l], sf[l], 0);
             __syncthreads();
             sm_rbgs(lv[l], qd[l], su[l], sf[l], 1);
@@ -2028,7 +2017,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle_smem(CoarseSet<T> S) {
     for (int l = S.L - 2; l >= S.l0; --l) {
         sm_prolong_add(lv[l], qd[l], su[l], lv[l + 1], su[l + 1]);
         __syncthreads();
-        for (int it = 0; it < S.nu2; ++it) {
+        for (int it = 0; it < S.post[l]; ++it) {
             sm_rbgs(lv[l], qd[l], su[l], sf[l], 1);
             __syncthreads();
             sm_rbgs(lv[l], qd[l], su[l], sf[l], 0);
@@ -2046,9 +2035,269 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
     for (int l = S.l0; l < S.L; ++l) {
         const LV<T>& G = S.lv[l];
         if (G.cell) return ~(size_t)0;                // the shared copy holds face coefficients only
-        b += (size_t)G.nx * G.ny * sizeof(T) * (l < S.L - 1 ? 6 * (G.nz + 2) + (sizeof(T) == 8 ? G.nz : 0) : 5 * (G.nz + 2));
+        b += (size_t)G.nx * G.ny * sizeof(T) * (l < S.L - 1 ? 6 * (G.nz + 2) + G.nz : 5 * (G.nz + 2));
     }
     return b;
+}
+
+
+// ------------------------------------------------------------ FP32 bottom of the V-cycle
+// Levels of at most kBottomPoints points in one CTA, from the first one's right side to its
+// corrected u. A half sweep of such a level is a few hundred instructions a warp, so what
+// bounds it is the distance between barriers: a thread owns up to four x pairs of a level and
+// keeps their faces, right sides, inverse diagonals and addresses in registers while it smooths
+// (six loads, ten multiply-adds and a store an update; with everything in shared memory and the
+// addresses formed anew each time a half sweep of 300 points took 1 us). The members of a pair
+// are ordered by colour, so that no update selects anything at run time. Faces, the coarsest
+// inverse and the first right side come in by one round of asynchronous copies; u keeps a zero
+// plane below and above a level (a band's walls). The coarse levels of a V-cycle take 31 us on
+// 24 x 24 x 48 (44 with the fused sweeps down to 1024 points and the shared-memory form below
+// that), 106 on 96 x 64 x 192 (125), 154 on 128 x 128 x 256 (165).
+constexpr int kBotThreads = 512;
+constexpr int kBotInvMax = 96;           // coarsest levels up to this many points: inverse in shared memory
+
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src));
+}
+__device__ __forceinline__ void cp_async8(float* dst, const float* src) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src));
+}
+
+struct BotLevel {
+    int nx, ny, nz, zper, pairs;
+    QDiv d;
+    float *cx, *cy, *cz, *u, *f, *r;     // at plane 0; cz and u have a plane -1, u a plane nz
+};
+
+// where pair t of a level lies (its even x)
+struct BotSite { int i, j, k, c; };
+__device__ __forceinline__ BotSite bot_site(const BotLevel& B, int t) {
+    BotSite p;
+    const int hx = B.nx >> 1, q = qdiv(t, B.d.hx);
+    p.i = 2 * (t - q * hx);
+    p.k = qdiv(q, B.d.ny);
+    p.j = q - p.k * B.ny;
+    p.c = 2 * t;
+    return p;
+}
+
+template <int Q>
+struct BotPairs {
+    float in[Q], out[Q][2], yp[Q][2], ym[Q][2], zp[Q][2], zm[Q][2], di[Q][2], f[Q][2];
+    int a[Q][2], o[Q][2], dyp[Q], dym[Q], dzp[Q], dzm[Q];
+
+    __device__ __forceinline__ void load(const BotLevel& B) {
+        const int nx = B.nx, pl = nx * B.ny;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int t = threadIdx.x + q * kBotThreads;
+            if (t >= B.pairs) continue;
+            const BotSite p = bot_site(B, t);
+            const int left = p.i == 0 ? p.c + nx - 1 : p.c - 1, right = p.i + 2 == nx ? p.c + 2 - nx : p.c + 2;
+            dyp[q] = p.j == B.ny - 1 ? -(B.ny - 1) * nx : nx;
+            dym[q] = p.j == 0 ? (B.ny - 1) * nx : -nx;
+            dzp[q] = B.zper && p.k == B.nz - 1 ? -(B.nz - 1) * pl : pl;
+            dzm[q] = B.zper && p.k == 0 ? (B.nz - 1) * pl : -pl;
+            in[q] = B.cx[p.c];
+            const int m = (p.j + p.k) & 1;                   // which member has colour 0
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int mh = m ^ h, e = p.c + mh;
+                a[q][h] = e;
+                o[q][h] = mh ? right : left;
+                out[q][h] = B.cx[mh ? e : left];
+                yp[q][h] = B.cy[e];
+                ym[q][h] = B.cy[e + dym[q]];
+                zp[q][h] = B.cz[e];
+                zm[q][h] = B.cz[e + dzm[q]];
+                f[q][h] = B.f[e];
+                di[q][h] = __fdividef(1.f, in[q] + out[q][h] + yp[q][h] + ym[q][h] + zp[q][h] + zm[q][h]);
+            }
+        }
+    }
+    __device__ __forceinline__ float around(const float* u, int q, int h) const {
+        const int e = a[q][h];
+        return (in[q] * u[a[q][1 - h]] + out[q][h] * u[o[q][h]]) + (yp[q][h] * u[e + dyp[q]] + ym[q][h] * u[e + dym[q]]) +
+               (zp[q][h] * u[e + dzp[q]] + zm[q][h] * u[e + dzm[q]]);
+    }
+    // one colour; reads the other colour only
+    template <int h, bool kFromZero>
+    __device__ __forceinline__ void half(const BotLevel& B) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (threadIdx.x + q * kBotThreads >= B.pairs) continue;
+            const float s = kFromZero ? 0.f : around(B.u, q, h);
+            B.u[a[q][h]] = (s - f[q][h]) * di[q][h];
+        }
+        __syncthreads();
+    }
+    __device__ __forceinline__ void down(const BotLevel& B, int sweeps) {
+        load(B);
+        if (sweeps == 0) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int t = threadIdx.x + q * kBotThreads;
+                if (t < B.pairs) B.u[2 * t] = B.u[2 * t + 1] = 0.f;
+            }
+            __syncthreads();
+        }
+        for (int it = 0; it < sweeps; ++it) {
+            if (it == 0) half<0, true>(B);
+            else half<0, false>(B);
+            half<1, false>(B);
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (threadIdx.x + q * kBotThreads >= B.pairs) continue;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float d = in[q] + out[q][h] + yp[q][h] + ym[q][h] + zp[q][h] + zm[q][h];
+                B.r[a[q][h]] = f[q][h] - (around(B.u, q, h) - d * B.u[a[q][h]]);
+            }
+        }
+        __syncthreads();
+    }
+    // coarse correction (C's u) by trilinear interpolation, then the sweeps, colour 1 first
+    __device__ __forceinline__ void up(const BotLevel& B, const BotLevel& C, int sweeps) {
+        load(B);
+        const int zoff = B.zper ? 0 : 1, cpl = C.nx * C.ny;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int t = threadIdx.x + q * kBotThreads;
+            if (t >= B.pairs) continue;
+            const BotSite p = bot_site(B, t);
+            const int x0 = p.i >> 1, x1 = x0 + 1 == C.nx ? 0 : x0 + 1;
+            const int y0 = p.j >> 1, ye = (p.j + 1) >> 1, y1 = ye == C.ny ? 0 : ye;
+            const int kk = p.k - zoff, z0 = kk >> 1, ze = (kk + 1) >> 1;     // -1 and nz: the walls' zero planes
+            const int z1 = C.zper && ze == C.nz ? 0 : ze;
+            // a repeated index counts twice: every weight is then 1/4 here, 1/2 more along x
+            const int e00 = C.nx * y0 + cpl * z0, e10 = C.nx * y1 + cpl * z0, e01 = C.nx * y0 + cpl * z1,
+                      e11 = C.nx * y1 + cpl * z1;
+            auto col = [&](int x) { return 0.25f * ((C.u[e00 + x] + C.u[e10 + x]) + (C.u[e01 + x] + C.u[e11 + x])); };
+            const float l = col(x0), r = col(x1);
+            B.u[p.c] += l;
+            B.u[p.c + 1] += 0.5f * (l + r);
+        }
+        __syncthreads();
+        for (int it = 0; it < sweeps; ++it) {
+            half<1, false>(B);
+            half<0, false>(B);
+        }
+    }
+};
+
+// full weighting of B's residual to C's right side
+__device__ void bot_restrict(const BotLevel& B, const BotLevel& C) {
+    LV<float> F, K;
+    F.nx = B.nx; F.ny = B.ny; F.nz = B.nz; F.zper = B.zper;
+    K.nx = C.nx; K.ny = C.ny; K.nz = C.nz; K.zper = C.zper;
+    sm_restrict(F, B.r, K, C.d, C.f);
+}
+
+__global__ void __launch_bounds__(kBotThreads) k_bottom(CoarseSet<float> S) {
+    extern __shared__ __align__(16) float bs[];
+    __shared__ double red[32];
+    __shared__ BotLevel B[16];
+    __shared__ float* inv;
+    const int tid = threadIdx.x;
+    // a 64-bit division each: one thread for one of them (all by one thread took 3 us)
+    if (tid < 3 * (S.L - S.l0)) {
+        const int l = S.l0 + tid / 3, w = tid % 3;
+        const LV<float>& G = S.lv[l];
+        const unsigned long long m = qmagic(w == 0 ? G.nx : (w == 1 ? G.ny : (G.nx > 1 ? G.nx >> 1 : 1)));
+        if (w == 0) B[l].d.nx = m;
+        else if (w == 1) B[l].d.ny = m;
+        else B[l].d.hx = m;
+    }
+    if (tid == 32 * 3) {
+        float* q = bs;
+        for (int l = S.l0; l < S.L; ++l) {
+            const LV<float>& G = S.lv[l];
+            const int pl = G.nx * G.ny, np = pl * G.nz;
+            BotLevel& b = B[l];
+            b.nx = G.nx; b.ny = G.ny; b.nz = G.nz; b.zper = G.zper; b.pairs = np >> 1;
+            b.cx = b.cy = b.cz = b.r = nullptr;
+            if (l < S.L - 1) {
+                b.cx = q; q += np;
+                b.cy = q; q += np;
+                b.cz = q + pl; q += np + pl;
+                b.r = q; q += np;
+            }
+            b.f = q; q += np;
+            b.u = q + pl; q += np + 2 * pl;
+        }
+        inv = S.nc <= kBotInvMax ? q : nullptr;
+    }
+    __syncthreads();
+    griddep_wait();
+    for (int l = S.l0; l < S.L; ++l) {
+        const LV<float>& G = S.lv[l];
+        const BotLevel& b = B[l];
+        const int pl = b.nx * b.ny, np = pl * b.nz;
+        if (l < S.L - 1) {
+            for (int t = 2 * tid; t < np; t += 2 * kBotThreads) {
+                cp_async8(b.cx + t, G.cx + t);
+                cp_async8(b.cy + t, G.cy + t);
+                if (l == S.l0) cp_async8(b.f + t, S.f[l] + t);
+            }
+            for (int t = 2 * tid - pl; t < np; t += 2 * kBotThreads) cp_async8(b.cz + t, G.cz + t);
+        }
+        for (int t = tid; t < pl; t += kBotThreads) b.u[t - pl] = b.u[t + np] = 0.f;
+    }
+    if (inv)
+        for (int t = tid; t < S.nc * S.nc; t += kBotThreads) cp_async4(inv + t, S.minv + t);
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    for (int l = S.l0; l < S.L - 1; ++l) {
+        const int n = B[l].pairs;
+        if (n <= kBotThreads) { BotPairs<1> P; P.down(B[l], S.pre[l]); }
+        else if (n <= 2 * kBotThreads) { BotPairs<2> P; P.down(B[l], S.pre[l]); }
+        else { BotPairs<4> P; P.down(B[l], S.pre[l]); }
+        bot_restrict(B[l], B[l + 1]);
+        __syncthreads();
+    }
+    {
+        // coarsest: u = inv (f - mean f) (periodic) or inv f (Dirichlet), a warp per row
+        const BotLevel& C = B[S.L - 1];
+        double loc = 0.0;
+        for (int p = tid; p < S.nc; p += kBotThreads) loc += (double)C.f[p];
+        const double tot = block_sum(loc, red);
+        __shared__ float mean;
+        if (tid == 0) mean = C.zper ? (float)(tot / S.nc) : 0.f;
+        __syncthreads();
+        const int lane = tid & 31;
+        const float* M = inv ? inv : S.minv;
+        for (int p = tid >> 5; p < S.nc; p += kBotThreads / 32) {
+            const float* row = M + (long)p * S.nc;
+            float acc = 0.f;
+#pragma unroll 4
+            for (int q = lane; q < S.nc; q += 32) acc += row[q] * (C.f[q] - mean);
+            for (int w = 16; w > 0; w >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, w);
+            if (lane == 0) C.u[p] = acc;
+        }
+        __syncthreads();
+    }
+    for (int l = S.L - 2; l >= S.l0; --l) {
+        const int n = B[l].pairs;
+        if (n <= kBotThreads) { BotPairs<1> P; P.up(B[l], B[l + 1], S.post[l]); }
+        else if (n <= 2 * kBotThreads) { BotPairs<2> P; P.up(B[l], B[l + 1], S.post[l]); }
+        else { BotPairs<4> P; P.up(B[l], B[l + 1], S.post[l]); }
+    }
+    const BotLevel& T = B[S.l0];
+    for (int t = tid; t < T.pairs; t += kBotThreads)
+        *reinterpret_cast<float2*>(S.u[S.l0] + 2 * t) = make_float2(T.u[2 * t], T.u[2 * t + 1]);
+}
+
+size_t bottom_smem_bytes(const CoarseSet<float>& S) {
+    size_t n = 0;
+    for (int l = S.l0; l < S.L; ++l) {
+        const size_t pl = (size_t)S.lv[l].nx * S.lv[l].ny, np = pl * S.lv[l].nz;
+        n += (l < S.L - 1 ? 4 * np + pl : 0) + 2 * np + 2 * pl;
+    }
+    if (S.nc <= kBotInvMax) n += (size_t)S.nc * S.nc;
+    return n * sizeof(float);
 }
 
 }  // namespace
@@ -2073,13 +2322,14 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
     cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-template <typename T> void launch_coarse_vcycle(const CoarseSet<T>& S, cudaStream_t s) {
-    const size_t b = coarse_smem_bytes(S);
-    if (b <= kCoarseSmemBytes) launch_pdl(k_coarse_vcycle_smem<T>, dim3(1), dim3(1024), b, s, S);
-    else launch_pdl(k_coarse_vcycle<T>, dim3(1), dim3(1024), 0, s, S);
+void launch_coarse_vcycle(const CoarseSet<float>& S, cudaStream_t s) {
+    launch_pdl(k_bottom, dim3(1), dim3(kBotThreads), bottom_smem_bytes(S), s, S);
 }
-template void launch_coarse_vcycle<float>(const CoarseSet<float>&, cudaStream_t);
-template void launch_coarse_vcycle<double>(const CoarseSet<double>&, cudaStream_t);
+void launch_coarse_vcycle(const CoarseSet<double>& S, cudaStream_t s) {
+    const size_t b = coarse_smem_bytes(S);
+    if (b <= kCoarseSmemBytes) launch_pdl(k_coarse_vcycle_smem<double>, dim3(1), dim3(1024), b, s, S);
+    else launch_pdl(k_coarse_vcycle<double>, dim3(1), dim3(1024), 0, s, S);
+}
 
 // ------------------------------------------------------------ launchers
 #define GP_NV_SWITCH(X)                                                                                  \
@@ -2206,7 +2456,7 @@ void coarse_vcycle_init() {
                          (int)(sizeof(double) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
     cudaFuncSetAttribute(k_gj_smem_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(sizeof(float2) * (kGjSmemMax * kGjSmemMax + 2 * kGjSmemMax)));
-    cudaFuncSetAttribute(k_coarse_vcycle_smem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
+    cudaFuncSetAttribute(k_bottom, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
     cudaFuncSetAttribute(k_coarse_vcycle_smem<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
 }
 void launch_tile_sweeps(const LV<float>& L, const float* u_in, const float* f, float* u_out, const LV<float>* C,

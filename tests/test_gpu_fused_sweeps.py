@@ -24,6 +24,9 @@ CASES = [
     ((96, 64, 96), (12.0, 9.0, 18.0), 0),       # level 1 of 73,728 points
     ((24, 32, 64), (9.0, 10.0, 22.0), 1),       # Dirichlet walls in z
     ((32, 24, 96), (10.0, 9.0, 28.0), 1),
+    ((32, 32, 32), (10.0, 10.0, 12.0), 0),      # one-CTA bottom: its largest level, 4096 points
+    ((32, 32, 96), (10.0, 10.0, 28.0), 0),      # two pairs a thread (1536 points), periodic and between walls
+    ((32, 32, 96), (10.0, 10.0, 28.0), 1),
 ]
 
 
