@@ -1945,8 +1945,8 @@ gp_status gp_set_vdw_radii(gp_ctx* c, const double* radii_dev, int n_atoms) {
             if (!(v > 0.0)) throw Err{GP_ERR_INVALID_ARG, "van der Waals radii must be positive"};
         if (n_atoms > c->rvdw_cap) {
             if (c->rvdw) cudaFree(c->rvdw);
-    if (c->ctab) cudaFree(c->ctab);
             c->rvdw = nullptr;
+            c->rvdw_cap = 0;
             if (cudaMalloc(&c->rvdw, sizeof(double) * n_atoms) != cudaSuccess) throw Err{GP_ERR_OOM, "cudaMalloc failed"};
             c->rvdw_cap = n_atoms;
         }
@@ -2346,6 +2346,7 @@ void gp_destroy(gp_ctx* c) {
     if (c->atoms) cudaFree(c->atoms);
     if (c->atoms32) cudaFree(c->atoms32);
     if (c->gtab) cudaFree(c->gtab);
+    if (c->ctab) cudaFree(c->ctab);
     if (c->gmtab) cudaFree(c->gmtab);
     if (c->gftab) cudaFree(c->gftab);
     if (c->rvdw) cudaFree(c->rvdw);
