@@ -182,21 +182,22 @@ def roofline_for(kind, prof, n0, hbm, hbm_src, prec_bytes):
     per_launch_s = p["ms"] / 1e3 / p["launches"]
     if kind == "smooth0":
         # FP32: one launch = one fused red-black sweep, 16 B/pt (read u, f, eps; write u);
-        # FP64: one launch = one colour of a sweep, half of 32 B/pt
-        bytes_per_launch = 16.0 * n0
+        # FP64: one launch = one colour of a sweep; every face once (24 B/pt), and u, f, 1/diagonal
+        # and the new u of half the points
+        bytes_per_launch = (16.0 if prec_bytes == 4 else 40.0) * n0
         achieved = bytes_per_launch / per_launch_s / 1e9
         out = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                "peak_source": hbm_src,
                "kernel": "k_rb_sweep (finest level, fused red-black sweep)" if prec_bytes == 4
-               else "k_rbgs (finest level, one colour)",
+               else "k_rbgs_pairs (finest level, one colour)",
                "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": per_launch_s * 1e3}
         if prec_bytes == 8:
-            # the FP64 colour sweep is bound by the FP64 pipe, not HBM: 30 FP64 flops per
-            # updated point (six face means, the weighted sum, the diagonal, the update)
-            gf = 30.0 * (n0 / 2) / per_launch_s / 1e9
+            # 13 FP64 flops per updated point: the weighted sum of six neighbours, f, and the
+            # product with the stored inverse diagonal
+            gf = 13.0 * (n0 / 2) / per_launch_s / 1e9
             out["fp64"] = {"achieved": gf, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
                            "frac": gf / FP64_PEAK_GFLOPS, "peak_source": "nominal FP64 (recipe table)",
-                           "flops_per_updated_point": 30}
+                           "flops_per_updated_point": 13}
         return out
     if kind == "res64":
         # read phi, rho, eps (FP64), write r in the working precision; 30 FP64 flops per point
