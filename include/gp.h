@@ -106,7 +106,8 @@ typedef struct {
     double beta;          /* kinds 1, 2: the exponent beta of Eq. 10 (2.4) */
     double zlim;          /* kind 2: z_lim of Eq. 19, Angstrom inside the cell (0) */
     int nu_coarse;        /* sweeps before and after the coarse correction on the second coarse level
-                             and below, 0 .. 8; the first coarse level and the finest use nu1, nu2;
+                             and below, and on a first coarse level of at most 4096 points, 0 .. 8;
+                             the finest level and a larger first coarse one use nu1, nu2;
                              0 = nu1, nu2 everywhere (4: those levels are cheap per sweep, and more
                              sweeps there cut the V-cycles per solve) */
     int inner_adapt;      /* full box: 1 = the first correction runs `inner` CG iterations, each later
