@@ -248,8 +248,10 @@ gp_status gp_residual6(gp_ctx* ctx, const double* rho_dev, const double* phi_dev
  * r = b - A6 phi - mu eps, b = -4 pi (rho - mean rho) (gp_get_stats has the
  * history). Method: flexible GMRES(restart) in FP64 on the field system with
  * the border eliminated, right-preconditioned by a V-cycle of the 7-point
- * multigrid in the context's precision (params.inner is not used). Uses the eps
- * of the last gp_set_dielectric. Errors: GP_ERR_INVALID_ARG (null array, tol <= 0),
+ * multigrid in the context's precision; if max_outer - 1 such cycles would not
+ * reach tol, by `inner` steps of multigrid-preconditioned CG for up to
+ * max_outer - 1 further ones. Uses the eps of the last gp_set_dielectric.
+ * Errors: GP_ERR_INVALID_ARG (null array, tol <= 0),
  * GP_ERR_STATE (no dielectric), GP_ERR_NOT_NEUTRAL, GP_ERR_NOT_CONVERGED /
  * GP_ERR_DIVERGED (phi holds the last iterate), GP_ERR_OOM (work fields are
  * allocated on first use), GP_ERR_CUDA. */

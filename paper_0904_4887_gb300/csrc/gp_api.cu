@@ -234,7 +234,7 @@ struct gp_ctx {
     std::vector<void*> misc;
     // sixth-order operator (Sec. III): D1 eps per axis, work fields
     double* f6_d1e = nullptr;      // 3 n: D1 eps, valid for eps_version f6_d1e_version
-    double* f6_r = nullptr;        // n: residual / operator output
+    double* f6_r = nullptr;        // n: the starting guess of a solve, the charge weights of the forces
     double* f6_w = nullptr;        // n: force weights
     double* f6_t3 = nullptr;       // 3 n: lam D1 phi per axis
     long eps_version = 0, f6_d1e_version = -1;
@@ -1293,7 +1293,13 @@ gp_status solve_impl(gp_ctx* c, const double* rho, double* phi, double tol) {
 // system alike. A7 differs from A6, so a better A7^-1 buys little: with 1, 2, 3, 5 and 7
 // steps of MG-preconditioned CG a solve of 64 x 64 x 128 points took 13, 11, 10, 10 and 10
 // GMRES steps, and 12.1, 12.8, 14.2, 18.8 and 23.9 ms with its adjoint and forces (17, 16,
-// 15, 15, 15 steps on 32 x 128 x 64). Device scalars used: 40..42 rho
+// 15, 15, 15 steps on 32 x 128 x 64). Where one V-cycle is a poor inverse (unequal spacings with one
+// sweep) and few vectors are kept, it stalls: on 32 x 64 x 32 points of 0.94 x 0.13 x 0.44 A with
+// nu1, nu2, nu_coarse, restart = 1, 0, 0, 2, 59 cycles end at the right side's own size, and 27 with
+// `inner` CG steps in its place end below 1e-10. So the solve goes over to those, for another
+// max_outer - 1 cycles, when its own have run out, or after a quarter of them would need more than
+// twice what is left (from the starting guess, kept in f6_r, unless they were fast). Device
+// scalars used: 40..42 rho
 // statistics, 44 sum of the last operator output, 45/46 sums of z and eps z,
 // 47 n, 48..50 eps statistics (48 = sum eps).
 constexpr int kS6Rho = 40, kS6Out = 44, kS6Z = 45, kS6N = 47, kS6Eps = 48;
@@ -1331,15 +1337,20 @@ void fd6_fix_constant(gp_ctx* c, double* z, bool transpose) {
     else launch_fd6_sub_ratio(c->n, z, nullptr, c->scal + kS6Z, c->scal + kS6N, c->s);
 }
 
+// strong: by `inner` steps of multigrid-preconditioned CG instead of one V-cycle
 template <typename T>
-void fd6_precondition(gp_ctx* c, const double* v, double* z, bool transpose) {
+void fd6_precondition(gp_ctx* c, const double* v, double* z, bool transpose, bool strong) {
     Hier<T>& F = full_hier<T>(c);
     {
         ProfScope ps(c, GP_PROF_MISC, 1);
         launch_cast_eps<T>(c->n, v, F.r, c->s);
     }
-    const long key = ((long)c->prm.nu_coarse << 32) | ((long)c->prm.nu1 << 8) | (long)c->prm.nu2;
-    run_graph(c, F.cycle_g, key, [&] { vcycle(c, F, F.x, F.r); });
+    if (strong) {
+        pcg<T>(c, F, c->prm.inner);
+    } else {
+        const long key = ((long)c->prm.nu_coarse << 32) | ((long)c->prm.nu1 << 8) | (long)c->prm.nu2;
+        run_graph(c, F.cycle_g, key, [&] { vcycle(c, F, F.x, F.r); });
+    }
     ProfScope ps(c, GP_PROF_MISC, 3);
     launch_fd6_to64<T>(c->n, F.x, c->eps64, z, c->partial, c->s);
     launch_finalize(c->partial, kReduceBlocks, 2, c->scal + kS6Z, c->s);
@@ -1390,11 +1401,14 @@ gp_status solve6_impl(gp_ctx* c, const double* rho, double* x, double tol, bool 
         ProfScope ps(c, GP_PROF_MISC, 3);
         fd6_fix_constant(c, x, transpose);           // the warm start onto the constraint
     }
+    GP_CUDA(cudaMemcpyAsync(c->f6_r, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->s));
     std::vector<double> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m + 1), hv(kMaxKrylov + 2);
     auto Hij = [&](int i, int j) -> double& { return H[(size_t)i * m + j]; };
-    double best = INFINITY, sum_out = 0.0;
+    double best = INFINITY, first = 1.0, sum_out = 0.0;
     gp_status result = GP_ERR_NOT_CONVERGED;
-    for (int cyc = 0; cyc < c->prm.max_outer; ++cyc) {
+    bool strong = false;
+    int left = c->prm.max_outer - 1;         // corrections this preconditioner may still make
+    for (int cyc = 0;; ++cyc) {
         // true residual, projected, into V0
         fd6_operator(c, x, rho, sb, -1.0, Vp(0), transpose);
         TVecList<double> V0;
@@ -1420,7 +1434,21 @@ gp_status solve6_impl(gp_ctx* c, const double* rho, double* x, double tol, bool 
         if (!std::isfinite(rn) || (cyc > 0 && rn > 1e3 * best)) { result = GP_ERR_DIVERGED; break; }
         best = std::min(best, rn);
         if (rn <= tol) { result = GP_OK; break; }
-        if (cyc == c->prm.max_outer - 1) break;
+        if (cyc == 0) first = rn;
+        else if (!strong) {
+            const double rate = std::log(rn / first) / cyc;              // of a cycle, on average
+            if (left == 0 || (4 * cyc >= c->prm.max_outer && std::log(tol / rn) < 2.0 * left * rate)) {
+                strong = true;
+                left = c->prm.max_outer - 1;
+                if (!(rate < -2.0)) {
+                    // from the start again: what a stalled GMRES leaves is what it is slow at
+                    best = INFINITY;
+                    GP_CUDA(cudaMemcpyAsync(x, c->f6_r, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->s));
+                    continue;
+                }
+            }
+        }
+        if (left-- == 0) break;
         {
             ProfScope ps(c, GP_PROF_KRYLOV, 1);
             launch_scale_by_norm<double>(n, Vp(0), Vp(0), c->scal + 15, c->s);
@@ -1430,7 +1458,7 @@ gp_status solve6_impl(gp_ctx* c, const double* rho, double* x, double tol, bool 
         g[0] = beta;
         int used = 0;
         for (int j = 0; j < m; ++j) {
-            fd6_precondition<T>(c, Vp(j), Zp(j), transpose);
+            fd6_precondition<T>(c, Vp(j), Zp(j), transpose, strong);
             fd6_operator(c, Zp(j), nullptr, 0.0, 1.0, Vp(j + 1), transpose);
             TVecList<double> V;
             V.n = j + 1;
