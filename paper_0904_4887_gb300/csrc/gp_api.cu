@@ -5,6 +5,7 @@
 #include "gp_common.cuh"
 
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -37,10 +38,13 @@ constexpr int kMaxInner = 16;   // PCG iterations one correction may take (adapt
 
 // A captured CUDA graph and what replaying it adds to the counters: the
 // kernel launches, V-cycles and inner iterations it holds, and (when it was
-// captured with profiling on) its event pairs per kernel group.
+// captured with profiling on) its event pairs per kernel group. It is captured
+// anew when anything the captured work depends on, its key, has changed.
+using GraphKey = std::array<long, 8>;
+
 struct GraphSlot {
     cudaGraphExec_t exec = nullptr;
-    long key = -1;
+    GraphKey key{};
     long launches = 0;
     int vcycles = 0, inner = 0;
     std::vector<int> kinds, nlaunch;
@@ -70,7 +74,8 @@ struct Hier {
     T* eps0 = nullptr;                          // owned level-0 cell eps (band only)
     T* x = nullptr; T* r = nullptr; T* p = nullptr; T* q = nullptr; T* z = nullptr;   // PCG, level 0
     T* tmp = nullptr;                           // level-0 ping-pong buffer of the fused sweep
-    int sweep_shape = -1;                       // tile shape chosen by the autotuner (-1: not yet)
+    int sweep_shape = -1;                       // tile shape in use: the caller's or the autotuner's
+    int tuned_shape = -1;                       // tile shape chosen by the autotuner (-1: not yet)
     T* minv = nullptr;
     int nc = 0;
     std::vector<void*> allocs;
@@ -250,7 +255,6 @@ struct gp_ctx {
     struct Pending { int kind; int launches; cudaEvent_t a, b; };
     std::vector<Pending> pending;
     std::vector<cudaEvent_t> event_pool;
-    long prm_on_key() const { return prof_on ? 1 : 0; }
     double prof_ms[GP_PROF_KINDS] = {};
     long prof_launches[GP_PROF_KINDS] = {};
     long prof_groups[GP_PROF_KINDS] = {};
@@ -486,12 +490,22 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
         c->stats.sweep_shape = H.sweep_shape;
     } else if (tile_finest(c, H)) {
         c->stats.sweep_shape = -1;
-    } else if (sizeof(T) == 4 && H.sweep_shape < 0) {
-        // smoother autotuner: time each tile shape on this level once
-        H.sweep_shape = rb_sweep_autotune<T>(H.lv[0], H.x, H.r, H.tmp, c->s);
-        GP_CHECK_LAUNCH();
+    } else if (sizeof(T) == 4) {
+        if (H.tuned_shape < 0) {
+            // smoother autotuner: time each tile shape on this level once
+            H.tuned_shape = rb_sweep_autotune<T>(H.lv[0], H.x, H.r, H.tmp, c->s);
+            GP_CHECK_LAUNCH();
+        }
+        H.sweep_shape = H.tuned_shape;
         c->stats.sweep_shape = H.sweep_shape;
     }
+}
+
+// what a captured V-cycle of H depends on, with up to three numbers of the caller's work around it
+template <typename T>
+GraphKey graph_key(const gp_ctx* c, const Hier<T>& H, long a = 0, long b = 0, long d = 0) {
+    const long smoother = tile_finest(c, H) ? -2 : H.sweep_shape;
+    return {c->prof_on ? 1L : 0L, smoother, c->prm.nu1, c->prm.nu2, c->prm.nu_coarse, a, b, d};
 }
 
 // ------------------------------------------------------------ V-cycle and PCG
@@ -664,12 +678,11 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
 // graph: captured once per key on the library stream, then replayed there,
 // ordered after and before the user's stream by events.
 template <typename F>
-void run_graph(gp_ctx* c, GraphSlot& g, long key, F&& body) {
+void run_graph(gp_ctx* c, GraphSlot& g, const GraphKey& key, F&& body) {
     if (!c->use_graphs) {
         body();
         return;
     }
-    key = key * 2 + (c->prof_on ? 1 : 0);
     if (!g.exec || g.key != key) {
         clear_slot(g);
         cudaStream_t user = c->s;
@@ -750,8 +763,7 @@ void pcg_body(gp_ctx* c, Hier<T>& H, int iters);
 // round trip) is one CUDA graph per hierarchy.
 template <typename T>
 void pcg(gp_ctx* c, Hier<T>& H, int iters) {
-    const long key = ((long)c->prm.nu_coarse << 32) | ((long)iters << 16) | ((long)c->prm.nu1 << 8) | (long)c->prm.nu2;
-    run_graph(c, H.pcg_g[iters <= kMaxInner ? iters : kMaxInner], key, [&] { pcg_body(c, H, iters); });
+    run_graph(c, H.pcg_g[iters <= kMaxInner ? iters : kMaxInner], graph_key(c, H, iters), [&] { pcg_body(c, H, iters); });
 }
 
 template <typename T>
@@ -953,9 +965,7 @@ template <typename T>
 void split_precondition(gp_ctx* c, int j, const T* v, T* z) {
     Hier<T>& B = band_hier<T>(c);
     if ((int)B.prec_g.size() <= j) B.prec_g.resize(j + 1);
-    const long key = ((long)c->prm.nu_coarse << 32) | ((long)c->prm.band_vcycles << 16) | ((long)c->prm.nu1 << 8) |
-                     (long)c->prm.nu2;
-    run_graph(c, B.prec_g[j], key, [&] { split_precondition_body<T>(c, v, z); });
+    run_graph(c, B.prec_g[j], graph_key(c, B, c->prm.band_vcycles), [&] { split_precondition_body<T>(c, v, z); });
 }
 
 // Right-preconditioned flexible GMRES(m) in the working precision T on
@@ -1170,9 +1180,7 @@ gp_status solve_impl(gp_ctx* c, const double* rho, double* phi, double tol) {
             F.solve_phi = phi;
             F.solve_rho = rho;
         }
-        const long key = ((long)c->prm.nu_coarse << 48) | ((long)use_df << 40) | ((long)k << 24) |
-                         ((long)c->prm.inner << 16) | ((long)c->prm.nu1 << 8) | c->prm.nu2;
-        run_graph(c, F.solve_g, key, [&] {
+        run_graph(c, F.solve_g, graph_key(c, F, k, c->prm.inner, use_df), [&] {
             for (int it = 0; it < k; ++it) {
                 if (it > 0) update_full(F.x);
                 outer_residual(F.r);
@@ -1348,8 +1356,7 @@ void fd6_precondition(gp_ctx* c, const double* v, double* z, bool transpose, boo
     if (strong) {
         pcg<T>(c, F, c->prm.inner);
     } else {
-        const long key = ((long)c->prm.nu_coarse << 32) | ((long)c->prm.nu1 << 8) | (long)c->prm.nu2;
-        run_graph(c, F.cycle_g, key, [&] { vcycle(c, F, F.x, F.r); });
+        run_graph(c, F.cycle_g, graph_key(c, F), [&] { vcycle(c, F, F.x, F.r); });
     }
     ProfScope ps(c, GP_PROF_MISC, 3);
     launch_fd6_to64<T>(c->n, F.x, c->eps64, z, c->partial, c->s);
