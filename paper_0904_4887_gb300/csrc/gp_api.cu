@@ -965,7 +965,8 @@ template <typename T>
 void split_precondition(gp_ctx* c, int j, const T* v, T* z) {
     Hier<T>& B = band_hier<T>(c);
     if ((int)B.prec_g.size() <= j) B.prec_g.resize(j + 1);
-    run_graph(c, B.prec_g[j], graph_key(c, B, c->prm.band_vcycles), [&] { split_precondition_body<T>(c, v, z); });
+    run_graph(c, B.prec_g[j], graph_key(c, B, c->prm.band_vcycles, c->band_first_interior),
+              [&] { split_precondition_body<T>(c, v, z); });
 }
 
 // Right-preconditioned flexible GMRES(m) in the working precision T on

@@ -53,3 +53,22 @@ def test_a_new_smoother_tile_is_the_one_that_runs(path, params):
         want.append(_launches(gp, f, path, pos, rho))
     assert want[0] != want[1]
     assert got == want
+
+
+def test_a_moved_dry_band():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0904_4887_gb300 import GPSolver
+    s = GPSolver(GRID, CELL, split=1)
+    steps, first = [], []
+    for k in (0, 9):
+        pos, gauss = _inputs(k * CELL[2] / GRID[2])
+        f = GPSolver(GRID, CELL, split=1)
+        for g in (s, f):
+            g.set_atoms(pos)
+            g.solve(g.build_rho(pos, gauss), tol=1e-10)
+            assert g.stats().split_active
+            steps.append(g.stats().vcycles)
+        first.append(s.stats().band_first)
+    assert first[1] == (first[0] + 9) % GRID[2]
+    assert max(steps) - min(steps) <= 2               # one GMRES step of two V-cycles, for rounding
