@@ -174,21 +174,25 @@ def make_inputs(w, frames, seed=0):
 
 
 # ----------------------------------------------------------------------------- GPU arm
-def roofline_for(kind, prof, n0, hbm, hbm_src, prec_bytes):
-    """Achieved vs peak for the kernel group `kind` from the live CUDA-event profile."""
+def roofline_for(kind, prof, n0, hbm, hbm_src, prec_bytes, shape=0):
+    """Achieved vs peak for the kernel group `kind` from the live CUDA-event profile; shape: the
+    smoother tile of the solve (gp_stats.sweep_shape)."""
     p = prof[kind]
     if p["launches"] == 0 or p["ms"] <= 0:
         return None
     per_launch_s = p["ms"] / 1e3 / p["launches"]
     if kind == "smooth0":
-        # FP32: one launch = one fused red-black sweep, 16 B/pt (read u, f, eps; write u);
+        # FP32: one launch = one fused red-black sweep, 16 B/pt (read u, f, eps; write u), or with
+        # tile -1 two of them from stored faces, 24 B/pt (read u, f, three faces; write u);
         # FP64: one launch = one colour of a sweep; every face once (24 B/pt), and u, f, 1/diagonal
         # and the new u of half the points
-        bytes_per_launch = (16.0 if prec_bytes == 4 else 40.0) * n0
+        tiles = prec_bytes == 4 and shape < 0
+        bytes_per_launch = (24.0 if tiles else 16.0 if prec_bytes == 4 else 40.0) * n0
         achieved = bytes_per_launch / per_launch_s / 1e9
         out = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                "peak_source": hbm_src,
-               "kernel": "k_rb_sweep (finest level, fused red-black sweep)" if prec_bytes == 4
+               "kernel": "k_tile_sweeps (finest level, two red-black sweeps)" if tiles
+               else "k_rb_sweep (finest level, fused red-black sweep)" if prec_bytes == 4
                else "k_rbgs_pairs (finest level, one colour)",
                "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_ms": per_launch_s * 1e3}
         if prec_bytes == 8:
@@ -308,7 +312,8 @@ def gpu_arm(args, rank, world):
     dominant = max(prof, key=lambda k: prof[k]["ms"])
     roof = roofline_for(dominant, prof, n0, hbm, hbm_src, prec_bytes) or {}
     npx = w.grid[0] // 2
-    shape_kernel = {0: "k_rb_sweep<float, 64, 8>", 1: "k_rb_sweep<float, 32, 16>", 2: "k_rb_sweep<float, 128, 4>",
+    shape_kernel = {-1: "k_tile_sweeps<2, 2>",
+                    0: "k_rb_sweep<float, 64, 8>", 1: "k_rb_sweep<float, 32, 16>", 2: "k_rb_sweep<float, 128, 4>",
                     3: "k_rb_sweep<float, 32, 8>", 4: "k_rb_sweep_rows<%d, 4>" % npx,
                     5: "k_rb_sweep_rows<%d, 6>" % npx, 6: "k_rb_sweep_rows<%d, 8>" % npx,
                     7: "k_rb_sweep_ws<%d, 6, 2>" % npx, 8: "k_rb_sweep_ws<%d, 4, 2>" % npx,
@@ -316,15 +321,16 @@ def gpu_arm(args, rank, world):
                     11: "k_rb_sweep_ws<%d, 16, 2>" % npx, 12: "k_rb_sweep_ws<%d, 14, 4>" % npx,
                     13: "k_rb_sweep_ws<%d, 14, 2>" % npx, 14: "k_rb_sweep_ws<%d, 12, 2>" % npx,
                     }.get(stats.sweep_shape, "k_rb_sweep")
-    # the smoother's roofline covers its ordinary sweeps (16 B/pt); the first sweep of each
-    # V-cycle starts from u = 0, reads no u (12 B/pt) and is timed in a group of its own
-    smooth = roofline_for("smooth0", prof, n0, hbm, hbm_src, prec_bytes)
+    # the smoother's roofline covers its ordinary launches (16 B/pt, tile -1 24); the first one of
+    # each V-cycle starts from u = 0, reads no u (4 B/pt less) and is timed in a group of its own
+    smooth = roofline_for("smooth0", prof, n0, hbm, hbm_src, prec_bytes, stats.sweep_shape)
     if smooth is not None and args.precision == 1 and prof.get("smooth0_zero", {}).get("launches"):
         z = prof["smooth0_zero"]
         z_s = z["ms"] / 1e3 / z["launches"]
-        smooth["from_zero"] = {"avg_launch_ms": z_s * 1e3, "algorithmic_bytes_per_launch": 12.0 * n0,
-                               "achieved": 12.0 * n0 / z_s / 1e9, "unit": "GB/s"}
-        smooth["kernel"] = shape_kernel + " (finest level, fused red-black sweep)"
+        z_bytes = smooth["algorithmic_bytes_per_launch"] - 4.0 * n0
+        smooth["from_zero"] = {"avg_launch_ms": z_s * 1e3, "algorithmic_bytes_per_launch": z_bytes,
+                               "achieved": z_bytes / z_s / 1e9, "unit": "GB/s"}
+        smooth["kernel"] = shape_kernel + smooth["kernel"][smooth["kernel"].index(" ("):]
         smooth["traffic"] = sweep_traffic(shape_kernel, w.name) if args.precision == 1 else None
     # the roofline object is the finest-level smoother's: the kernel with the largest share of the
     # step's device time in the launch list (a kernel group such as the coarse levels, made of many
@@ -376,7 +382,8 @@ def gpu_arm(args, rank, world):
             out["phases"] = {k: {"ms_per_step": v["ms"] / ncmp, "share": v["ms"] / tot if tot else 0.0}
                              for k, v in pv.items() if v["launches"]}
             out["smoother"] = roofline_for("smooth0", pv, n0 if not sst.split_active else
-                                           int(round(n_full * sst.wet_fraction)), hbm, hbm_src, pb)
+                                           int(round(n_full * sst.wet_fraction)), hbm, hbm_src, pb,
+                                           sst.sweep_shape)
             out["residual64"] = roofline_for("res64", pv, n_full, hbm, hbm_src, pb)
         if sv is not solver:
             del sv

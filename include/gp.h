@@ -365,7 +365,8 @@ enum {
     GP_PROF_FORCES_EPS = 2,  /* dielectric (solvent) force */
     GP_PROF_FORCES_RHO = 3,  /* charge-motion force */
     GP_PROF_RES64 = 4,       /* FP64 full-box residual + norm (outer correction) */
-    GP_PROF_SMOOTH0 = 5,     /* red-black Gauss-Seidel on the finest multigrid level */
+    GP_PROF_SMOOTH0 = 5,     /* red-black Gauss-Seidel on the finest multigrid level (with sweep_shape
+                                -1 in gp_stats two sweeps a launch, the coarse correction added in the first) */
     GP_PROF_MG_FINE = 6,     /* finest-level residual, restriction, prolongation */
     GP_PROF_MG_COARSE = 7,   /* all coarser levels and the coarsest solve */
     GP_PROF_KRYLOV = 8,      /* CG operator application, dot products, updates */
@@ -374,7 +375,7 @@ enum {
     GP_PROF_MISC = 11,       /* reductions, gauge, atom wrapping */
     GP_PROF_UPDATE64 = 12,   /* FP64 phi update */
     GP_PROF_ENERGY = 13,     /* energy reductions */
-    GP_PROF_SMOOTH0_ZERO = 14, /* the first finest-level sweep of a V-cycle, from u = 0 (reads no u) */
+    GP_PROF_SMOOTH0_ZERO = 14, /* the first finest-level launch of a V-cycle, from u = 0 (reads no u) */
     GP_PROF_KINDS = 15
 };
 

@@ -594,12 +594,13 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
         } else if (tiled(l)) {
             if constexpr (sizeof(T) == 4) {
                 const int nu = pre_of(l);
-                ProfScope ps(c, l == 0 ? GP_PROF_MG_FINE : GP_PROF_MG_COARSE, (nu + 1) / 2 + 1);
                 for (int it = 0; it < nu; it += 2) {
+                    ProfScope ps(c, l > 0 ? GP_PROF_MG_COARSE : (it == 0 ? GP_PROF_SMOOTH0_ZERO : GP_PROF_SMOOTH0), 1);
                     T* to = it == 0 ? u : other(l, cur[l]);
                     launch_tile_sweeps(V, it == 0 ? nullptr : cur[l], f, to, nullptr, nullptr, std::min(2, nu - it), 0, c->s);
                     cur[l] = to;
                 }
+                ProfScope ps(c, l == 0 ? GP_PROF_MG_FINE : GP_PROF_MG_COARSE, 1);
                 launch_residual_restrict(V, cur[l], f, H.lv[l + 1], H.f[l + 1], c->s);
             }
             continue;
@@ -646,7 +647,7 @@ void vcycle(gp_ctx* c, Hier<T>& H, T* u0, const T* f0) {
         if (tiled(l)) {
             if constexpr (sizeof(T) == 4) {
                 const int nu = post_of(l);
-                ProfScope ps(c, l == 0 ? GP_PROF_MG_FINE : GP_PROF_MG_COARSE, (nu + 1) / 2);
+                ProfScope ps(c, l == 0 ? GP_PROF_SMOOTH0 : GP_PROF_MG_COARSE, (nu + 1) / 2);
                 for (int it = 0; it < nu; it += 2) {
                     T* to = other(l, cur[l]);
                     launch_tile_sweeps(V, cur[l], f, to, it == 0 ? &H.lv[l + 1] : nullptr, cur[l + 1], std::min(2, nu - it),
