@@ -33,6 +33,10 @@ struct Err {
 #define GP_CHECK_LAUNCH() GP_CUDA(cudaGetLastError())
 
 constexpr long kTileFinest = 120000;   // finest levels up to this size take the fused sweeps
+// FP64 grids up to this size store the finest level's faces and inverse diagonal, 32 bytes a point: at
+// 5.4e8 points a sixth-order solve then takes 200 GB. Above it they could be what does not fit
+// (1024 x 1024 x 768 points: 300 GB of 298), and the sweeps form the coefficients from eps.
+constexpr long kStoredFaces = 1L << 29;
 constexpr long kTinyLevel = 4096;      // a first coarse level up to this size takes nu_coarse sweeps
 constexpr int kMaxInner = 16;   // PCG iterations one correction may take (adaptive counts included)
 
@@ -69,7 +73,7 @@ struct Hier {
     T* cy[16] = {};
     T* cz[16] = {};
     T* dinv[16] = {};
-    LV<T> fine;                                 // level 0 as the sweeps and products see it (FP64: stored faces)
+    LV<T> fine;                                 // level 0 as the sweeps and products see it (FP64: stored faces, if any)
     LV<T> tile0;                                // level 0 with stored faces, for the fused sweeps (small FP32 grids)
     T* eps0 = nullptr;                          // owned level-0 cell eps (band only)
     T* x = nullptr; T* r = nullptr; T* p = nullptr; T* q = nullptr; T* z = nullptr;   // PCG, level 0
@@ -374,7 +378,7 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
             L.ihx2 = (T)(1.0 / (hx * hx)); L.ihy2 = (T)(1.0 / (hy * hy)); L.ihz2 = (T)(1.0 / (hz * hz));
             L.cell = (l == 0);
             L.eps = nullptr; L.cx = L.cy = L.cz = L.dinv = nullptr;
-            if (l > 0 || sizeof(T) == 8 || (long)lx * ly * lz <= kTileFinest) {
+            if (l > 0 || (long)lx * ly * lz <= (sizeof(T) == 8 ? kStoredFaces : kTileFinest)) {
                 H.cx[l] = alloc_level(H, lx, ly, lz);
                 H.cy[l] = alloc_level(H, lx, ly, lz);
                 H.cz[l] = alloc_level(H, lx, ly, lz);
@@ -410,7 +414,7 @@ void alloc_hier(gp_ctx* c, Hier<T>& H, int nx, int ny, int nz, int zper, int lev
     if (H.cx[0]) {
         H.tile0.cell = 0;
         H.tile0.cx = H.cx[0]; H.tile0.cy = H.cy[0]; H.tile0.cz = H.cz[0]; H.tile0.dinv = H.dinv[0];
-        if (sizeof(T) == 8) H.fine = H.tile0;
+        if (sizeof(T) == 8) H.fine = H.tile0;      // without faces: lv[0], its coefficients from eps
     }
 }
 
@@ -455,15 +459,14 @@ void coarse_coeffs(gp_ctx* c, Hier<T>& H) {
         launch_coarsen_faces<T>(F, C.nx, C.ny, C.nz, H.cx[l], H.cy[l], H.cz[l], c->s);
         GP_CHECK_LAUNCH();
     }
-    if (sizeof(T) == 4 && H.cx[0]) {
+    // the finest level's faces where its sweeps read them (FP64: with the inverse diagonal)
+    if (sizeof(T) == 8 ? H.cx[0] != nullptr : tile_finest(c, H)) {
         ProfScope ps(c, GP_PROF_SETUP, 1);
-        launch_cell_faces<T>(H.lv[0], H.cx[0], H.cy[0], H.cz[0], nullptr, c->s);
+        launch_cell_faces<T>(H.lv[0], H.cx[0], H.cy[0], H.cz[0], H.dinv[0], c->s);
         GP_CHECK_LAUNCH();
     }
-    // FP64: the finest level's faces, and every level's inverse diagonal
     if (sizeof(T) == 8) {
-        ProfScope ps(c, GP_PROF_SETUP, 2);
-        launch_cell_faces<T>(H.lv[0], H.cx[0], H.cy[0], H.cz[0], H.dinv[0], c->s);
+        ProfScope ps(c, GP_PROF_SETUP, 1);
         launch_diag_inverse<T>(H.lv, H.dinv, 1, levels - 1, c->s);
         GP_CHECK_LAUNCH();
     }

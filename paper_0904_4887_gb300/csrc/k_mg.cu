@@ -114,7 +114,8 @@ int grid_for(long n, int threads) {
 
 // ------------------------------------------------------------ smoothing
 // Red-black Gauss-Seidel half sweep for A u = f: u_i = (sum c u_nb - f_i) / sum c.
-// One thread per x-pair; it updates the member of the pair with the colour.
+// One thread per x-pair; it updates the member of the pair with the colour. Coefficients
+// from eps: the finest FP64 level of grids too large to store its faces.
 template <typename T>
 __global__ void k_rbgs(LV<T> L, T* u, const T* f, int color, int init) {
     griddep_wait();
@@ -2421,13 +2422,15 @@ void launch_update_phi(const Geo& g, double* phi, const T* e_full, const T* e_ba
 }
 
 template <typename T> void launch_rbgs(const LV<T>& L, T* u, const T* f, int color, cudaStream_t s, bool init) {
-    if (!L.cell && (sizeof(T) == 4 || L.dinv)) {
+    if (sizeof(T) == 4 || !L.cell) {
         const long pairs = (long)(L.nx / 2) * L.ny * L.nz;
         launch_pdl(k_rbgs_pairs<T>, dim3(grid_for(pairs, 256)), dim3(256), 0, s, L, u, f, color, (int)init);
         return;
     }
-    const long rows = (long)L.ny * L.nz;
-    launch_pdl(k_rbgs<T>, dim3(row_blocks(rows)), dim3(row_threads(L.nx / 2)), 0, s, L, u, f, color, (int)init);
+    if constexpr (sizeof(T) == 8) {
+        const long rows = (long)L.ny * L.nz;
+        launch_pdl(k_rbgs<T>, dim3(row_blocks(rows)), dim3(row_threads(L.nx / 2)), 0, s, L, u, f, color, (int)init);
+    }
 }
 template <typename T> void launch_residual(const LV<T>& L, const T* u, const T* f, T* r, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
