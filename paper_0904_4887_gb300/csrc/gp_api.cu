@@ -1576,12 +1576,17 @@ double gamma_cutoff(const Geo& g, double se, double tail) {
 //
 // The line to the direct sum: that one drops the images beyond the tail radius, and so does
 // far's transform up to a ripple of the size of one term there, so tails looser than 1e-12
-// stay direct; and a grid too coarse for the K that brings rn below three quarters of the
-// radius gains nothing. Everywhere else the split is the faster one, down to the smallest
+// stay direct. So do tails below 1e-14 with beta < 1/2, where eps follows gamma^(2 beta) with
+// an unbounded slope at zero: far carries an absolute error of about 1e-16 wherever gamma is
+// small, the direct sum of positive terms a relative one (beta = 1/4, a tail of 1e-16 and solvent
+// 100 A deep: eps is off by 2.6e-9 of its largest value through the series and 5e-10 direct; at the
+// default tail both by 1.6e-8, and at beta = 0.4 both by 2e-14). And a grid too coarse for the K
+// that brings rn below three quarters of the radius gains nothing, nor does one with an extent
+// above 512, for which the band-limited transforms have no instance. Everywhere else the split is the faster one, down to the smallest
 // grids (24 x 24 x 48 with 24 atoms: 0.50 + 0.45 ms against 3.3 + 2.5, whose blocks are few).
 bool plan_far(gp_ctx* c, const DielParams& dp, int n_atoms, double se, double tail) {
     const Geo& g = c->g;
-    if (tail > 1e-12 || !fft_static_extents(g)) return false;
+    if (tail > 1e-12 || (tail < 1e-14 && dp.beta2 < 1.0) || !fft_static_extents(g)) return false;
     const double two_pi = 2.0 * kPi;
     GammaFar f{};
     f.bx = two_pi / g.lx; f.by = two_pi / g.ly; f.bz = two_pi / g.lz;
