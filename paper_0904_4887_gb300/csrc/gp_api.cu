@@ -1603,7 +1603,7 @@ bool plan_far(gp_ctx* c, const DielParams& dp, int n_atoms, double se, double ta
         else hi = mid;
     }
     f.rn = hi;
-    if (f.rn > 25.0 || f.rn > 0.75 * dp.rcut) return false;
+    if (f.rn > kNearMax || f.rn > 0.75 * dp.rcut) return false;
     f.mx = std::min((int)(f.K / f.bx), g.nx / 2 - 1);
     f.my = std::min((int)(f.K / f.by), g.ny / 2 - 1);
     f.mz = std::min((int)(f.K / f.bz), g.nz / 2 - 1);

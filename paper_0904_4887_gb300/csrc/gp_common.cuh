@@ -185,8 +185,9 @@ __host__ __device__ inline long plane_of(int nx, int ny) { return (long)nx * ny;
 // switching-function tables (k_fields.cu): s and h = s'/(s d) as polynomials in q = d^2
 constexpr int kSwNI = 512, kSwDeg = 7;
 // Packed FP32 copies, kSwVec float4 per interval: the kSwSplit lowest coefficients as
-// hi/lo pairs, then the rest as single floats (they are small enough that FP32 leaves
-// < 1e-14 relative). From interval s_tail on (u = (d - r0)/w >= 4) s is within 7.7e-9 of
+// hi/lo pairs, then the rest as single floats: s within 1e-14, h within 3e-13 of itself at its
+// table's inner end, where s'/d is 1e-5 of its peak (with six pairs at half the intervals and degree 9 the
+// force's error against 64 bits was the same or larger, 2.5e-12 against 2.4e-12). From interval s_tail on (u = (d - r0)/w >= 4) s is within 7.7e-9 of
 // one: there the row holds 1 - s as single floats.
 constexpr int kSwSplit = 4, kSwVec = 3;
 struct SwTables {
@@ -257,6 +258,7 @@ constexpr int kFarIv = 256, kFarDeg = 9;    // table of far's transform: interva
 constexpr int kNearIv = 1024;               // tables of near(d) and -near'(d)/d: intervals of d^2 in [0, rn^2]
 constexpr int kNearDeg = 7, kNearSplit = 4; // their polynomials' degree; coefficients held as float pairs
 constexpr int kNearVec = 3;                 // float4 per interval: 4 pairs, 4 singles
+constexpr int kNearMax = 25;                // largest near radius, Angstrom
 constexpr int kNearDirect = 16;             // intervals below this: near(d) by its formula (the square root's cusp)
 struct GammaFar {
     double K, d0, s, rn, rcut;

@@ -1330,10 +1330,13 @@ __global__ void k_gamma_tables(Geo g, Atoms at, DielParams p, const double* rvdw
 
 // ----------------------------------------------------------------- the split sum's near part
 // near(d) = exp(-d) (1 - w(d)) (k_gfar.cu) of a pair from its squared distance x = d^2/dq in
-// table units, held as a float pair: interval (int)x, local variable t in [-1, 1], a degree-9
+// table units, held as a float pair: interval (int)x, local variable t in [-1, 1], a degree-7
 // polynomial (Chebyshev; its first kNearSplit coefficients and its last steps in df).
 // The intervals below kNearDirect (d < rn/8), where the square root's branch point spoils
 // polynomials, take exp(-d) by its table and subtract far(d) < 2e-9, which FP32 gives.
+// kNearRows: the rows exp(-n) those distances use.
+constexpr int kNearRows = 4;
+static_assert(kNearDirect * 64 == kNearIv && kNearRows * 8 > kNearMax && kNearRows <= kGT1, "d < rn/8 <= kNearMax/8 < kNearRows");
 constexpr int kNearSmem = kNearIv * kNearVec * (int)sizeof(float4);
 __device__ __forceinline__ void near_table(float* dst, const float4* src) {
     for (int q = threadIdx.x; q < kNearVec * kNearIv; q += blockDim.x) reinterpret_cast<float4*>(dst)[q] = __ldg(src + q);
@@ -1489,7 +1492,7 @@ __global__ void __launch_bounds__(TT, 2) k_build_eps_gamma_df(Geo g, Atoms at, D
         };
         const int total = block_compact(0, nq, keep, nullptr, scratch);
         const int win = total <= GCAP ? nq : GCAP;
-        constexpr int nrow = 4, ns = NS + nrow;          // the direct branch has d < 3
+        constexpr int ns = NS + kNearRows;
         for (int w0 = 0; w0 < nq; w0 += win) {
             const int m = block_compact(w0, min(w0 + win, nq), keep, elist, scratch);
             for (int e0 = 0; e0 < m; e0 += GB) {
@@ -1507,7 +1510,7 @@ __global__ void __launch_bounds__(TT, 2) k_build_eps_gamma_df(Geo g, Atoms at, D
                         else if (c < TX + TY) sy2[e][c - TX] = sq;
                         else sz2[e][c - TX - TY] = sq;
                     } else {
-                        // rows 0 .. 3: exp(rvdw - n); row 0 alone scales the table's terms
+                        // rows exp(rvdw - n); row 0 alone scales the table's terms
                         const int n = c - NS;
                         srow[e][n] = df_mul(as_df(gt.at[a].a), as_df(__ldg(gt.t1 + n)));
                         if (n == 0) skz[e] = gf.up && gt.at[a].kzl > 0 ? kzs : 0;
@@ -1840,7 +1843,7 @@ __global__ void __launch_bounds__(TT) k_forces_eps_gamma_df(Geo g, Atoms at, Die
                     wq[warp][c] = df_mul(df_mul(dd, dd), idq);
                 }
                 const df A = as_df(gt.at[a].a);
-                if (lane < 4) wrow[warp][lane] = df_mul(A, as_df(__ldg(gt.t1 + lane)));
+                if (lane < kNearRows) wrow[warp][lane] = df_mul(A, as_df(__ldg(gt.t1 + lane)));
                 __syncwarp();
                 near_pairs(gf.up && gt.at[a].kzl > 0 ? kzs : 0, A, dq);
             }

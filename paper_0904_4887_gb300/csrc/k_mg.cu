@@ -1558,13 +1558,14 @@ __global__ void k_band_eps(Geo g, const T* eps, int first, int band_nz, T* beps)
     }
 }
 
-// f_band = r - A e_vac on the band's interior planes (full-box operator, periodic)
+// dst = src^-1/2 (the vacuum solve's factors of the split)
 template <typename T>
 __global__ void k_rsqrt(long n, const T* src, T* dst) {
     for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x)
         dst[t] = rsqrt(src[t]);
 }
 
+// f_band = r - A e_vac on the band's interior planes (full-box operator, periodic)
 template <typename T>
 __global__ void k_band_rhs(Geo g, const T* eps, const T* r, const T* ev, int first, int band_nz, T* fb) {
     const long pl = plane_of(g.nx, g.ny);
@@ -2045,10 +2046,12 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
 // ------------------------------------------------------------ FP32 bottom of the V-cycle
 // Levels of at most kBottomPoints points in one CTA, from the first one's right side to its
 // corrected u. A half sweep of such a level is a few hundred instructions a warp, so what
-// bounds it is the distance between barriers: a thread owns up to four x pairs of a level and
-// keeps their faces, right sides, inverse diagonals and addresses in registers while it smooths
-// (six loads, ten multiply-adds and a store an update; with everything in shared memory and the
-// addresses formed anew each time a half sweep of 300 points took 1 us). The members of a pair
+// bounds it is the distance between barriers (issue slots 22 to 26% used, most waits at barriers and
+// on loads): a thread owns up to four x pairs of a level and loads their faces, right sides,
+// inverse diagonals and addresses once for all its sweeps (six loads, ten multiply-adds and a
+// store an update; with everything in shared memory and the addresses formed anew each time a half
+// sweep of 300 points took 1 us). One pair and two stay in the 128 registers a thread has; four, on
+// levels above 2048 points, do not: 628 bytes of a thread are spilled. The members of a pair
 // are ordered by colour, so that no update selects anything at run time. Faces, the coarsest
 // inverse and the first right side come in by one round of asynchronous copies; u keeps a zero
 // plane below and above a level (a band's walls). The coarse levels of a V-cycle take 31 us on
