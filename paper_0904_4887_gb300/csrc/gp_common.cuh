@@ -425,13 +425,13 @@ template <typename T> void launch_update_p(const LV<T>& L, T* p, const T* z, con
 template <typename T> void launch_copy_level(const LV<T>& L, T* dst, const T* src, cudaStream_t s);
 
 // the bottom of a V-cycle in one CTA (k_mg.cu): levels l0 .. L-1
-// Levels up to this size run in the persistent kernel: in FP32 what a thread's registers hold
-// (with the line at 1024 points instead, and the fused sweeps above it, a step on 24 x 24 x 48 takes
-// 1.25 ms instead of 1.20, on 96 x 64 x 192 2.75 instead of 2.67). In FP64 the
-// kernel is bound by its one SM's FP64 pipe: a half sweep of 2048 points takes 2.5 us there, a
-// launch across the SMs 3.5 us; of 4096 points 5 us and 3.5 us.
-constexpr int kBottomPoints = 4096;
-template <typename T> constexpr int coarse_block_points() { return sizeof(T) == 8 ? 2048 : kBottomPoints; }
+// Levels up to this size run in the persistent kernel. FP32: with levels of up to 4096 points in it
+// (four pairs a thread, beyond its registers) a step on 24 x 24 x 48 points, whose level 1 holds 3456,
+// takes 1.26 ms instead of 1.22, one on 32^3 (4096) 1.43 instead of 1.35; with the line at 1024 and the
+// fused sweeps above it, 1.49 instead of 1.39 on 24^3 and 1.78 instead of 1.67 on 48^3 (levels of 1728).
+// FP64: the kernel is bound by its one SM's FP64 pipe: a half sweep of 2048 points takes 2.5 us
+// there, a launch across the SMs 3.5 us; of 4096 points 5 us and 3.5 us.
+constexpr int kBottomPoints = 2048;
 template <typename T>
 struct CoarseSet {
     int l0, L, nc;

@@ -2047,17 +2047,17 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
 // Levels of at most kBottomPoints points in one CTA, from the first one's right side to its
 // corrected u. A half sweep of such a level is a few hundred instructions a warp, so what
 // bounds it is the distance between barriers (issue slots 22 to 26% used, most waits at barriers and
-// on loads): a thread owns up to four x pairs of a level and loads their faces, right sides,
-// inverse diagonals and addresses once for all its sweeps (six loads, ten multiply-adds and a
+// on loads): a thread owns one or two x pairs of a level and keeps their faces, right sides,
+// inverse diagonals and addresses in registers while it smooths (six loads, ten multiply-adds and a
 // store an update; with everything in shared memory and the addresses formed anew each time a half
-// sweep of 300 points took 1 us). One pair and two stay in the 128 registers a thread has; four, on
-// levels above 2048 points, do not: 628 bytes of a thread are spilled. The members of a pair
+// sweep of 300 points took 1 us; four pairs spilled 628 bytes of a thread). The members of a pair
 // are ordered by colour, so that no update selects anything at run time. Faces, the coarsest
 // inverse and the first right side come in by one round of asynchronous copies; u keeps a zero
 // plane below and above a level (a band's walls). The coarse levels of a V-cycle take 31 us on
 // 24 x 24 x 48 (44 with the fused sweeps down to 1024 points and the shared-memory form below
 // that), 106 on 96 x 64 x 192 (125), 154 on 128 x 128 x 256 (165).
 constexpr int kBotThreads = 512;
+static_assert(kBottomPoints <= 4 * kBotThreads, "two pairs a thread");
 constexpr int kBotInvMax = 96;           // coarsest levels up to this many points: inverse in shared memory
 
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
@@ -2257,8 +2257,7 @@ __global__ void __launch_bounds__(kBotThreads) k_bottom(CoarseSet<float> S) {
     for (int l = S.l0; l < S.L - 1; ++l) {
         const int n = B[l].pairs;
         if (n <= kBotThreads) { BotPairs<1> P; P.down(B[l], S.pre[l]); }
-        else if (n <= 2 * kBotThreads) { BotPairs<2> P; P.down(B[l], S.pre[l]); }
-        else { BotPairs<4> P; P.down(B[l], S.pre[l]); }
+        else { BotPairs<2> P; P.down(B[l], S.pre[l]); }
         bot_restrict(B[l], B[l + 1]);
         __syncthreads();
     }
@@ -2286,8 +2285,7 @@ __global__ void __launch_bounds__(kBotThreads) k_bottom(CoarseSet<float> S) {
     for (int l = S.L - 2; l >= S.l0; --l) {
         const int n = B[l].pairs;
         if (n <= kBotThreads) { BotPairs<1> P; P.up(B[l], B[l + 1], S.post[l]); }
-        else if (n <= 2 * kBotThreads) { BotPairs<2> P; P.up(B[l], B[l + 1], S.post[l]); }
-        else { BotPairs<4> P; P.up(B[l], B[l + 1], S.post[l]); }
+        else { BotPairs<2> P; P.up(B[l], B[l + 1], S.post[l]); }
     }
     const BotLevel& T = B[S.l0];
     for (int t = tid; t < T.pairs; t += kBotThreads)
