@@ -2053,9 +2053,9 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
 // sweep of 300 points took 1 us; four pairs spilled 628 bytes of a thread). The members of a pair
 // are ordered by colour, so that no update selects anything at run time. Faces, the coarsest
 // inverse and the first right side come in by one round of asynchronous copies; u keeps a zero
-// plane below and above a level (a band's walls). The coarse levels of a V-cycle take 31 us on
-// 24 x 24 x 48 (44 with the fused sweeps down to 1024 points and the shared-memory form below
-// that), 106 on 96 x 64 x 192 (125), 154 on 128 x 128 x 256 (165).
+// plane below and above a level (a band's walls). The coarse levels of a V-cycle, this kernel and the
+// fused sweeps above it, take 118 us on 96 x 64 x 192 (profiled; 125 with the shared-memory form below
+// and launches per half sweep above) and 150 on 128 x 128 x 256 (165).
 constexpr int kBotThreads = 512;
 static_assert(kBottomPoints <= 4 * kBotThreads, "two pairs a thread");
 constexpr int kBotInvMax = 96;           // coarsest levels up to this many points: inverse in shared memory
