@@ -1282,12 +1282,12 @@ gp_status solve_impl(gp_ctx* c, const double* rho, double* phi, double tol) {
             // FP32 (or FP64) flexible GMRES on the correction equation A e = r,
             // preconditioned by the dry/wet split; the FP64 outer loop couples
             // the two regions through the full-box residual. It reduces the residual as far
-            // as its precision allows, or to a tenth of the tolerance where that is less, and ends
-            // between that and a hundredth (a step gains a decade): on the FP64 96 x 96 x 192 slab at tol
-            // 1e-10, 5e-13 to 1.2e-12 of b in 17.1 ms, phi off by 2e-13 to 1.4e-12. With 0.003 in place of
-            // 0.1, 6e-14, 3e-14 and 18.5 ms; to the full 1e-7, 3e-14, 1.5e-14 and 21.4 ms. A caller who
-            // needs the smaller error asks for the smaller tol
-            fgmres_inner<T>(c, rT, ekry, c->prm.restart, std::max(sizeof(T) == 4 ? 1e-4 : 1e-7, 0.1 * tol / rn));
+            // as its precision allows, or to a thousandth of the tolerance where that is less: with
+            // the scaled vacuum solve a step gains a decade, and the full 1e-7 in FP64 went on to the
+            // rounding of the solution (64-bit 96 x 96 x 192 slab at tol 1e-10: 3e-14 of b, 21.4 ms; 6e-14 and
+            // 18.5 ms here). A tenth of the tolerance, 17.1 ms, ends at 5e-13 to 1e-11: over 16 slabs
+            // forces were off by up to 100 times what a correction to 1e-7 (1e-4 in FP32) leaves
+            fgmres_inner<T>(c, rT, ekry, c->prm.restart, std::max(sizeof(T) == 4 ? 1e-4 : 1e-7, 1e-3 * tol / rn));
         } else if (split) {
             {
                 ProfScope ps(c, GP_PROF_FFT, 5);
