@@ -2046,7 +2046,7 @@ size_t coarse_smem_bytes(const CoarseSet<T>& S) {
 // ------------------------------------------------------------ FP32 bottom of the V-cycle
 // Levels of at most kBottomPoints points in one CTA, from the first one's right side to its
 // corrected u. A half sweep of such a level is a few hundred instructions a warp, so what
-// bounds it is the distance between barriers (issue slots 22 to 26% used, most waits at barriers and
+// bounds it is the distance between barriers (issue slots 19 to 22% used, most waits at barriers and
 // on loads): a thread owns one or two x pairs of a level and keeps their faces, right sides,
 // inverse diagonals and addresses in registers while it smooths (six loads, ten multiply-adds and a
 // store an update; with everything in shared memory and the addresses formed anew each time a half
